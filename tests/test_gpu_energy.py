@@ -1,0 +1,50 @@
+"""The energy sums and bound statistics on random fields, against the oracle: 2D and 3D, ragged and
+small grids (fewer points than a block), both precisions."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import band as obm  # noqa: E402
+from oracle import model as omodel  # noqa: E402
+from paper_2606_04347_gb300 import Plan  # noqa: E402
+from paper_2606_04347_gb300 import workloads as wl  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _params(n, prec):
+    dim = 2 if n[2] == 1 else 3
+    return wl.workload("c2", n=16)[0].replace(dim=dim, n=n, model=0, precision=prec, cg_rtol=1e-13 if prec == 0 else 1e-6)
+
+
+def _membrane(p, kind, rng):
+    if kind == "full":      # every point in the band, g between 0.46 and 1.125
+        return rng.uniform(0.2, 0.8, size=p.shape)
+    r = np.sqrt(sum(c ** 2 for c in wl.grid(p.n, p.half_len, p.dim)))
+    eps = {"shell": 0.25, "thin": 0.09}[kind]
+    return wl.tanh_profile(1.6 - r, eps) * np.ones(p.shape)
+
+
+@pytest.mark.parametrize("prec,tol", [(0, 1e-11), (1, 3e-6)])
+@pytest.mark.parametrize("n,kind", [((8, 8, 1), "full"), ((96, 64, 1), "shell"), ((32, 16, 8), "full"), ((64, 32, 32), "shell")])
+def test_energy_sums_match_oracle(n, kind, prec, tol):
+    """Every sum of Eq. (2.16) on random fields.  FP32: g, W(u) and f(u) carry a few FP32
+    roundings (below 1e-6 relative, all terms positive but the mass, whose square enters), the
+    sums themselves none."""
+    p = _params(n, prec).replace(gamma=20.0, M=30.0, ubar=0.3)
+    rng = np.random.default_rng(5)
+    dt = np.float64 if prec == 0 else np.float32
+    phi = _membrane(p, kind, rng).astype(dt).astype(np.float64)
+    u = rng.uniform(0.2, 0.9, size=p.shape).astype(dt).astype(np.float64)
+    band, G = obm.band_mask(phi, p.band_mask_hi), omodel.g_loc(phi)
+    want = omodel.energy(u, G, band, p, rtol=1e-13)
+    plan = Plan(p)
+    dev = lambda a: torch.tensor(a, dtype=plan.dtype, device=DEV)  # noqa: E731
+    d = plan.energy(dev(phi), dev(u))
+    assert abs(d["energy"] - want["total"]) <= tol * abs(want["total"])
+    assert abs(d["mass"] - want["mass"]) <= tol * abs(want["mass"])
+    mb, lo, hi = omodel.bound_stats(u, G, p.recover_delta)
+    assert d["band_size"] == band.sum() and (d["max_bound"], d["umin"], d["umax"]) == (mb, lo, hi)
+    assert abs(d["volume"] - omodel.volume(phi, p)) <= 1e-13 * phi.sum()
