@@ -359,6 +359,7 @@ etd_status etd_plan_batch(const etd_params* params, int nruns, void* cuda_stream
         if (it == tuned.end()) it = tuned.emplace(key, autotune(params[i], b->origin)).first;
         r.tile = it->second;
       }
+      r.tile.shared = nruns > 1;
       ETD_CUDA(cudaStreamCreateWithFlags(&r.stream, cudaStreamNonBlocking));
       ETD_CUDA(cudaEventCreateWithFlags(&r.done, cudaEventDisableTiming));
       r.plan = make_plan(r.params, r.stream, r.tile);

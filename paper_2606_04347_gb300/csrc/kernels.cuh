@@ -873,13 +873,15 @@ static __global__ void k_band_scatter(long long n, const unsigned char* __restri
 // flux across the band edge); (A v)_i = sum_faces c (v_i - v_q).  Vectors are compact
 // (length M, band order), so every CG phase streams contiguous arrays.
 template <typename T> struct CGVec {
-  T *x, *r, *u, *p, *q;   // compact vectors; q holds s = A p
-  T* r1;                  // second residual buffer (the multigrid iterations alternate r, r1)
-  T* idg;                 // inverse diagonal
+  T *x, *r, *p, *q;       // compact vectors of the solve
+  float *b, *e, *o, *t;   // level-0 vectors of the multigrid cycle
+  float* idg;             // inverse diagonal
   T* c;                   // face coefficients, c[d * cap + i], d = x+, x-, y+, y-, z+, z-
+  float* c32;             // the same for the multigrid cycle, times csc (FP32 storage: c itself)
   __half* c16;            // the same in FP16 for the multigrid sweeps (FP32 storage only, else null)
   int* nb;                // compact index of the face neighbour (i itself when absent)
   int cap;
+  T csc;                  // FP64 storage: a power of two near h^2, which takes c32 to order one
 };
 
 template <typename T>
@@ -893,7 +895,7 @@ __global__ void k_cg_setup(Geo g, ModelC<T> mc, const int* __restrict__ idx, con
     const Nb n = neighbours(g, p);
     const int q[6] = {n.xp, n.xm, n.yp, n.ym, n.zp, n.zm};
     const T gc = G[p];
-    T d = 0;
+    float d = 0;
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       T c = 0;
@@ -903,11 +905,13 @@ __global__ void k_cg_setup(Geo g, ModelC<T> mc, const int* __restrict__ idx, con
         j = bmap[q[f]];
       }
       v.c[f * v.cap + i] = c;
-      if (v.c16) v.c16[f * v.cap + i] = __float2half_rn((float)c);
+      const float cf = sizeof(T) == 4 ? (float)c : (float)(c * v.csc);
+      if (sizeof(T) == 8) v.c32[f * v.cap + i] = cf;
+      if (v.c16) v.c16[f * v.cap + i] = __float2half_rn(cf);
       v.nb[f * v.cap + i] = j;
-      d += c;
+      d += cf;
     }
-    v.idg[i] = d > (T)0 ? (T)1 / d : (T)1;
+    v.idg[i] = d > 0.0f ? 1.0f / d : 1.0f;
   }
 }
 
@@ -1188,34 +1192,7 @@ static __global__ void k_cc_down(CCLevels lv, const int* __restrict__ ccL, const
   acc.end();
 }
 
-template <typename T>
-__device__ __forceinline__ T band_apply(const CGVec<T>& v, const T* __restrict__ a, int i) {
-  const T ai = __ldcg(a + i);
-  T s = 0;
-#pragma unroll
-  for (int f = 0; f < 6; ++f) s += v.c[f * v.cap + i] * (ai - __ldcg(a + v.nb[f * v.cap + i]));
-  return s;
-}
-
-// Right-hand sides f of the band solve.
-template <typename T> struct RhsField {
-  const T* f;
-  __device__ double operator()(long long p) const { return (double)f[p]; }
-};
-template <typename T> struct RhsGU {  // G (u - ubar): coupled nonlocal operand (Eq. (1.2))
-  const T* G;
-  const T* u;
-  double ubar;
-  __device__ double operator()(long long p) const { return (double)G[p] * ((double)u[p] - ubar); }
-};
-template <typename T> struct RhsGF {  // G f(u): fixed-model operand (Eq. (2.16))
-  const T* G;
-  const T* u;
-  __device__ double operator()(long long p) const { return (double)G[p] * (double)find(u[p]); }
-};
-
 struct CGCtl {
-  double* acc;          // 16 FP64 accumulators (zeroed before launch)
   unsigned* bar;        // [0] monotonic arrival count
   int* status;          // plan status word
   int* iters;           // out: iterations
@@ -1227,14 +1204,13 @@ struct CGCtl {
   const int* ncomp;     // connected band components (device)
   const int* comp;      // component of each band node
   const double* csize;  // nodes per component
-  double* csum;         // 2 kCompCap FP64 accumulators (zeroed before launch): f, then x
+  double* csum;         // 2 kCompCap FP64 accumulators (zeroed by the solve): f, then x
 };
 
-// Inside the band CG kernel every vector that the kernel itself writes (x, r, u, p, q and
-// the multigrid levels' b, e, o, t) is read with __ldcg: an L2 load, never the read-only
-// path that a const __restrict__ pointer would allow, which is only valid for data that no
-// thread writes during the launch.  The couplings, neighbour lists and level maps are built
-// by earlier launches and are read normally.
+// Inside the band solve every global vector that the kernel itself writes is read with __ldcg:
+// an L2 load, never the read-only path that a const __restrict__ pointer would allow, which is
+// only valid for data that no thread writes during the launch.  The couplings, neighbour lists
+// and level maps are built by earlier launches and are read normally.
 
 // Grid-wide barrier for a cooperative launch on one monotonic arrival counter (zeroed
 // before the launch): barrier number e completes when the counter reaches e * gridDim.x,
@@ -1261,19 +1237,25 @@ __device__ __forceinline__ bool grid_sync(const CGCtl& c) {
   __shared__ int ok;
   if (threadIdx.x == 0) {
     const unsigned nb = gridDim.x;
+    // the status word is read along with the counter, not after it (one L2 latency less); a
+    // failure that this misses is seen at the next barrier, whose poll looks at it too
+    int st = *(volatile int*)c.status;
     const unsigned old = atom_add_acq_rel_gpu(c.bar, 1u);
     const unsigned target = (old / nb + 1u) * nb;
     if (old + 1u != target) {
       const long long t0 = clock64();
-      while ((int)(ld_acquire_gpu(c.bar) - target) < 0) {
+      for (;;) {
+        st = *(volatile int*)c.status;
+        if ((int)(ld_acquire_gpu(c.bar) - target) >= 0 || st != 0) break;
         if (clock64() - t0 > c.budget) {
           atomicCAS(c.status, 0, 6);
+          st = 6;
           break;
         }
         __nanosleep(32);
       }
     }
-    ok = (*(volatile int*)c.status == 0);
+    ok = st == 0;
   }
   __syncthreads();
   return ok;
@@ -1290,32 +1272,6 @@ __device__ __forceinline__ bool grid_sync(const CGCtl& c) {
 // degree-2 Chebyshev polynomial in D^-1 A (the two sweeps commute, so the cycle stays
 // symmetric), and the coarsest level takes an even number of sweeps with the same pair.
 constexpr int kMGMax = 7;
-
-template <typename T> struct MGL {
-  const int* cnt;      // node count (device)
-  const int* list;     // flat cell index of each node on this level's grid
-  const T* c;          // couplings c[f * cap + i]
-  const int* nb;       // neighbour node of each face (i itself when absent)
-  const T* idg;        // inverse diagonal
-  int cap;
-  const int* agg;      // parent node on level l+1 (l < nlev-1)
-  const int* child;    // child[k * cap + I]: node of level l-1 in sub-cell k, -1 if none (l >= 1)
-  T* b;                // right-hand side (level 0: the CG residual r)
-  T* e;                // pre-smoothed correction
-  T* o;                // output correction (level 0: the preconditioned residual u)
-  T* t;                // scratch: residual handed to the restriction, first post-sweep
-};
-
-template <typename T> struct MGP {
-  int nlev;            // 1 = plain Jacobi
-  int gl;              // levels 0..gl-1 are processed by the whole grid, the rest by block 0
-  int csweeps;         // Jacobi sweeps on the coarsest level (even)
-  int nu;              // pre- and post-smoothing sweeps (1 or 2)
-  T w1, w2;            // Jacobi weights of the first and second sweep (one Chebyshev pair)
-  T alpha;             // over-correction of the coarse-grid correction
-  const __half* c16;   // level-0 couplings in FP16 for the sweeps (null: use L[0].c)
-  MGL<T> L[kMGMax];
-};
 
 // Multigrid set-up steps, written for any grid-stride partition (t0, ns) so that the large
 // levels run them as grid-wide kernels and the small ones all inside one block.
@@ -1345,17 +1301,16 @@ __device__ __forceinline__ void mg_parent_body(const int* __restrict__ list, int
 }
 
 // Galerkin couplings of level l from level l-1.
-template <typename T>
 __device__ __forceinline__ void mg_coarse_body(const int* __restrict__ clist, int M, Ext ec, int is3d,
                                                const unsigned char* __restrict__ fmark,
                                                const int* __restrict__ fmap, Ext ef,
-                                               const T* __restrict__ fc, int fcap, const int* __restrict__ cmap,
-                                               T* __restrict__ c, int* __restrict__ nb, T* __restrict__ idg,
+                                               const float* __restrict__ fc, int fcap, const int* __restrict__ cmap,
+                                               float* __restrict__ c, int* __restrict__ nb, float* __restrict__ idg,
                                                int* __restrict__ child, int cap, int t0, int ns) {
   for (int I = t0; I < M; I += ns) {
     const int C = clist[I];
     const int X = C % ec.x, tq = C / ec.x, Y = tq % ec.y, Z = tq / ec.y;
-    T s[6] = {0, 0, 0, 0, 0, 0};
+    float s[6] = {0, 0, 0, 0, 0, 0};
     // the 8 children's marks, then their indices, then their couplings: three rounds of
     // independent loads instead of a dependent chain per child
     int Fk[8], jk[8];
@@ -1383,14 +1338,14 @@ __device__ __forceinline__ void mg_coarse_body(const int* __restrict__ clist, in
     const int zp = Z + 1 == ec.z ? 0 : Z + 1, zm = Z == 0 ? ec.z - 1 : Z - 1;
     const int ncell[6] = {(Z * ec.y + Y) * ec.x + xp, (Z * ec.y + Y) * ec.x + xm, (Z * ec.y + yp) * ec.x + X,
                           (Z * ec.y + ym) * ec.x + X, (zp * ec.y + Y) * ec.x + X, (zm * ec.y + Y) * ec.x + X};
-    T d = 0;
+    float d = 0;
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       c[f * cap + I] = s[f];
-      nb[f * cap + I] = s[f] > (T)0 ? cmap[ncell[f]] : I;
+      nb[f * cap + I] = s[f] > 0.0f ? cmap[ncell[f]] : I;
       d += s[f];
     }
-    idg[I] = d > (T)0 ? (T)1 / d : (T)1;
+    idg[I] = d > 0.0f ? 1.0f / d : 1.0f;
   }
 }
 
@@ -1404,44 +1359,43 @@ static __global__ void k_mg_parent(const int* __restrict__ list, const int* __re
   mg_parent_body(list, *cnt, f, is3d, c, cmap, agg, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-template <typename T>
-__global__ void k_mg_coarse(const int* __restrict__ clist, const int* __restrict__ ccnt, Ext ec, int is3d,
+static __global__ void k_mg_coarse(const int* __restrict__ clist, const int* __restrict__ ccnt, Ext ec, int is3d,
                             const unsigned char* __restrict__ fmark, const int* __restrict__ fmap, Ext ef,
-                            const T* __restrict__ fc, int fcap, const int* __restrict__ cmap, T* __restrict__ c,
-                            int* __restrict__ nb, T* __restrict__ idg, int* __restrict__ child, int cap) {
-  mg_coarse_body<T>(clist, *ccnt, ec, is3d, fmark, fmap, ef, fc, fcap, cmap, c, nb, idg, child, cap,
+                            const float* __restrict__ fc, int fcap, const int* __restrict__ cmap, float* __restrict__ c,
+                            int* __restrict__ nb, float* __restrict__ idg, int* __restrict__ child, int cap) {
+  mg_coarse_body(clist, *ccnt, ec, is3d, fmark, fmap, ef, fc, fcap, cmap, c, nb, idg, child, cap,
                     blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // One level's arrays for the single-block set-up of the small levels.
-template <typename T> struct MGSetLevel {
+struct MGSetLevel {
   Ext e;
   int cap;
   int* cnt;
   int* list;
   int* map;
   unsigned char* mark;
-  T* c;
+  float* c;
   int* nb;
-  T* idg;
+  float* idg;
   int* agg;
   int* child;
 };
 
-template <typename T> struct MGSetTail {
+struct MGSetTail {
   int first, nlev, is3d;
-  MGSetLevel<T> L[kMGMax];
+  MGSetLevel L[kMGMax];
 };
 
 // Levels first..nlev-1 built in order by one block of 1024 threads: mark, compact (one
 // contiguous chunk of cells per thread, block-wide exclusive scan), parent map of the
 // finer level, Galerkin couplings.  The finer level of `first` is complete on entry.
-template <typename T> __global__ void __launch_bounds__(1024) k_mg_setup_tail(MGSetTail<T> a) {
+static __global__ void __launch_bounds__(1024) k_mg_setup_tail(MGSetTail a) {
   __shared__ int part[1024];
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int l = a.first; l < a.nlev; ++l) {
-    const MGSetLevel<T>& F = a.L[l - 1];
-    const MGSetLevel<T>& L = a.L[l];
+    const MGSetLevel& F = a.L[l - 1];
+    const MGSetLevel& L = a.L[l];
     for (int i = tid; i < L.cap; i += nt) L.mark[i] = 0;
     __syncthreads();
     const int MF = *F.cnt;
@@ -1471,503 +1425,10 @@ template <typename T> __global__ void __launch_bounds__(1024) k_mg_setup_tail(MG
     __syncthreads();
     const int M = part[nt - 1];
     mg_parent_body(F.list, MF, F.e, a.is3d, L.e, L.map, F.agg, tid, nt);
-    mg_coarse_body<T>(L.list, M, L.e, a.is3d, F.mark, F.map, F.e, F.c, F.cap, L.map, L.c, L.nb,
+    mg_coarse_body(L.list, M, L.e, a.is3d, F.mark, F.map, F.e, F.c, F.cap, L.map, L.c, L.nb,
                       L.idg, L.child, L.cap, tid, nt);
     __syncthreads();
   }
-}
-
-template <typename T> __device__ __forceinline__ T mg_apply(const MGL<T>& L, const T* __restrict__ v, int i) {
-  const T vi = __ldcg(v + i);
-  T s = 0;
-#pragma unroll
-  for (int f = 0; f < 6; ++f) s += L.c[f * L.cap + i] * (vi - __ldcg(v + L.nb[f * L.cap + i]));
-  return s;
-}
-
-// Barrier between consecutive V-cycle phases: a grid barrier when either phase runs on the
-// whole grid, a block barrier inside block 0 when both run on block 0 alone.  The first
-// call is free: the caller has already synchronised the grid.
-struct PhaseSync {
-  bool prev, first;
-  __device__ bool step(bool cur, const CGCtl& c) {
-    const bool g = prev || cur;
-    prev = cur;
-    if (first) {
-      first = false;
-      return true;
-    }
-    if (g) return grid_sync(c);
-    if (blockIdx.x == 0) __syncthreads();
-    return true;
-  }
-};
-
-// A level-0 coupling for the multigrid sweeps: the FP16 copy where there is one (the
-// preconditioner tolerates its rounding; the CG operator itself keeps the FP32 couplings).
-template <typename T>
-__device__ __forceinline__ T mg_coef(const T* __restrict__ c, const __half* __restrict__ h, int k) {
-  return h ? (T)__half2float(h[k]) : c[k];
-}
-
-// The CG update x += a p, r_new = r_old - a q folded into the first smoothing sweep of the
-// V-cycle that preconditions r_new (the sweep needs r_new at the neighbours, which it
-// recomputes from r_old and q there, so the separate update pass and its barrier go away).
-template <typename T> struct CGFuse {
-  bool on;
-  const T* rold;
-  T* x;
-  const T* p;
-  const T* q;
-  T a;
-  double* rr;       // accumulates (r_new, r_new)
-  double tol2;      // stop when (r_new, r_new) <= tol2
-  double* zero;     // a CG accumulator every block has finished reading: zeroed on the way
-};
-
-// u = V(b), one symmetric V(nu,nu) cycle (nu = 1 or 2 weighted-Jacobi sweeps before and
-// after the coarse-grid correction, which is scaled by alpha) for the level-0 right-hand
-// side b.  On entry b is complete and visible (or, with the fused CG update, r_old, q, p and
-// x are); on return every block has written its share of u (level-0 o) and added its part of
-// (b,u) to *ru.  Residuals of the pre-sweeps are carried algebraically: e1 = w D^-1 b,
-// r1 = b - A e1 (needs b at the neighbours), e2 = e1 + w D^-1 r1, r2 = r1 - w A D^-1 r1
-// (needs r1 at the neighbours).  Returns -1 if a barrier failed, 1 if the fused update met
-// the tolerance (the cycle is abandoned, *rr_out holds (r_new, r_new)), else 0.
-template <typename T>
-__device__ __forceinline__ int mg_vcycle(const MGP<T>& mg, const CGCtl& c, T* __restrict__ b0, const CGFuse<T>& F, double* ru,
-                         double* rr_out) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-  PhaseSync ps{true, true};
-  const T w1 = mg.w1, w2 = mg.w2, al = mg.alpha;
-  // after the barrier that follows the fused sweep: every block sees (r_new, r_new)
-  auto fused_check = [&]() -> bool {
-    const double rr = *(volatile double*)F.rr;
-    *rr_out = rr;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *F.zero = 0.0;
-    return rr <= F.tol2;
-  };
-  for (int l = 0; l < mg.nlev - 1; ++l) {
-    const MGL<T>& L = mg.L[l];
-    const MGL<T>& Cl = mg.L[l + 1];
-    bool grid = l < mg.gl;
-    int t0 = grid ? tid : threadIdx.x, ns = grid ? nth : blockDim.x;
-    if (!ps.step(grid, c)) return -1;
-    if (grid || blockIdx.x == 0) {
-      T* __restrict__ r1out = mg.nu == 2 ? L.o : L.t;
-      const T* __restrict__ Lidg = L.idg;
-      const T* __restrict__ Lc = L.c;
-      const __half* __restrict__ Lh = l == 0 ? mg.c16 : nullptr;
-      const int* __restrict__ Lnb = L.nb;
-      T* __restrict__ Le = L.e;
-      const int M = *L.cnt, cap = L.cap;
-      if (l == 0 && F.on) {
-        const T* __restrict__ Ro = F.rold;
-        const T* __restrict__ Q = F.q;
-        const T* __restrict__ P = F.p;
-        T* __restrict__ X = F.x;
-        const T a = F.a;
-        T rr = 0;  // per-thread partial in the storage precision (a few nodes per thread)
-        for (int i = t0; i < M; i += ns) {
-          const T bi = __ldcg(Ro + i) - a * __ldcg(Q + i);
-          X[i] = __ldcg(X + i) + a * __ldcg(P + i);
-          b0[i] = bi;
-          rr += bi * bi;
-          const T ei = w1 * Lidg[i] * bi;
-          T s = 0;
-#pragma unroll
-          for (int f = 0; f < 6; ++f) {
-            const int j = Lnb[f * cap + i];
-            // FP32 couplings here: this sweep is gather-bound and the half loads measured slower
-            s += Lc[f * cap + i] * (ei - w1 * Lidg[j] * (__ldcg(Ro + j) - a * __ldcg(Q + j)));
-          }
-          Le[i] = ei;
-          r1out[i] = bi - s;
-        }
-        block_add((double)rr, F.rr);
-      } else {
-        const T* __restrict__ Lb = l == 0 ? b0 : L.b;
-#pragma unroll 2
-        for (int i = t0; i < M; i += ns) {
-          const T bi = __ldcg(Lb + i);
-          const T ei = w1 * Lidg[i] * bi;
-          T s = 0;
-#pragma unroll
-          for (int f = 0; f < 6; ++f) {
-            const int j = Lnb[f * cap + i];
-            s += mg_coef(Lc, Lh, f * cap + i) * (ei - w1 * Lidg[j] * __ldcg(Lb + j));
-          }
-          Le[i] = ei;
-          r1out[i] = bi - s;
-        }
-      }
-      if (mg.nu == 2) {  // the second sweep accumulates into the coarse right-hand side
-        const int Mc = *Cl.cnt;
-        for (int I = t0; I < Mc; I += ns) Cl.b[I] = 0;
-      }
-    }
-    if (mg.nu == 2) {
-      // second sweep e2 = e1 + w D^-1 r1, its residual r2 = r1 - w A D^-1 r1 added to the
-      // parent aggregate's right-hand side (the restriction of piecewise-constant P)
-      if (!ps.step(grid, c)) return -1;
-      if (l == 0 && F.on && fused_check()) return 1;
-      if (grid || blockIdx.x == 0) {
-        const T* __restrict__ Lo = L.o;
-        const T* __restrict__ Lidg = L.idg;
-        const T* __restrict__ Lc = L.c;
-        const __half* __restrict__ Lh = l == 0 ? mg.c16 : nullptr;
-        const int* __restrict__ Lnb = L.nb;
-        const int* __restrict__ Lagg = L.agg;
-        T* __restrict__ Le = L.e;
-        T* Cb = Cl.b;
-        const int M = *L.cnt, cap = L.cap;
-#pragma unroll 2
-        for (int i = t0; i < M; i += ns) {
-          const T oi = __ldcg(Lo + i);
-          const T di = Lidg[i] * oi;
-          T s = 0;
-#pragma unroll
-          for (int f = 0; f < 6; ++f) {
-            const int j = Lnb[f * cap + i];
-            s += mg_coef(Lc, Lh, f * cap + i) * (di - Lidg[j] * __ldcg(Lo + j));
-          }
-          Le[i] = __ldcg(Le + i) + w2 * di;
-          atomicAdd(Cb + Lagg[i], oi - w2 * s);
-        }
-      }
-      continue;
-    }
-    grid = (l + 1) < mg.gl;
-    t0 = grid ? tid : threadIdx.x;
-    ns = grid ? nth : blockDim.x;
-    if (!ps.step(grid, c)) return -1;
-    if (l == 0 && F.on && fused_check()) return 1;
-    if (grid || blockIdx.x == 0) {
-      const int M = *Cl.cnt;
-      for (int I = t0; I < M; I += ns) {
-        T s = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int j = Cl.child[q * Cl.cap + I];
-          if (j >= 0) s += __ldcg(L.t + j);
-        }
-        Cl.b[I] = s;
-      }
-    }
-  }
-  {
-    const MGL<T>& L = mg.L[mg.nlev - 1];
-    const bool grid = (mg.nlev - 1) < mg.gl;
-    const int t0 = grid ? tid : threadIdx.x, ns = grid ? nth : blockDim.x;
-    if (!ps.step(grid, c)) return -1;
-    if (grid || blockIdx.x == 0) {
-      const int M = *L.cnt;
-      for (int i = t0; i < M; i += ns) L.e[i] = w1 * L.idg[i] * __ldcg(L.b + i);
-    }
-    for (int s = 1; s < mg.csweeps; ++s) {
-      if (!ps.step(grid, c)) return -1;
-      const T* src = (s & 1) ? L.e : L.o;
-      T* dst = (s & 1) ? L.o : L.e;
-      if (grid || blockIdx.x == 0) {
-        const int M = *L.cnt;
-        for (int i = t0; i < M; i += ns) dst[i] = __ldcg(src + i) + ((s & 1) ? w2 : w1) * L.idg[i] * (__ldcg(L.b + i) - mg_apply(L, src, i));
-      }
-    }
-  }
-  for (int l = mg.nlev - 2; l >= 0; --l) {
-    const MGL<T>& L = mg.L[l];
-    const MGL<T>& Cl = mg.L[l + 1];
-    const bool grid = l < mg.gl;
-    const int t0 = grid ? tid : threadIdx.x, ns = grid ? nth : blockDim.x;
-    if (!ps.step(grid, c)) return -1;
-    T acc = 0;
-    if (grid || blockIdx.x == 0) {
-      T* __restrict__ out = mg.nu == 2 ? L.t : L.o;
-      const T* __restrict__ Le = L.e;
-      const T* __restrict__ Co = Cl.o;
-      const T* __restrict__ Lb = l == 0 ? b0 : L.b;
-      const T* __restrict__ Lidg = L.idg;
-      const T* __restrict__ Lc = L.c;
-      const __half* __restrict__ Lh = l == 0 ? mg.c16 : nullptr;
-      const int* __restrict__ Lnb = L.nb;
-      const int* __restrict__ Lagg = L.agg;
-      const int M = *L.cnt, cap = L.cap;
-#pragma unroll 2
-      for (int i = t0; i < M; i += ns) {
-        const T ei = __ldcg(Le + i) + al * __ldcg(Co + Lagg[i]);
-        T s = 0;
-#pragma unroll
-        for (int f = 0; f < 6; ++f) {
-          const int j = Lnb[f * cap + i];
-          s += mg_coef(Lc, Lh, f * cap + i) * (ei - (__ldcg(Le + j) + al * __ldcg(Co + Lagg[j])));
-        }
-        const T bi = __ldcg(Lb + i);
-        const T o1 = ei + (mg.nu == 2 ? w2 : w1) * Lidg[i] * (bi - s);
-        out[i] = o1;
-        if (l == 0 && mg.nu == 1) acc += bi * o1;
-      }
-    }
-    if (mg.nu == 2) {
-      if (!ps.step(grid, c)) return -1;
-      if (grid || blockIdx.x == 0) {
-        const T* __restrict__ Lt = L.t;
-        const T* __restrict__ Lb = l == 0 ? b0 : L.b;
-        const T* __restrict__ Lidg = L.idg;
-        const T* __restrict__ Lc = L.c;
-        const __half* __restrict__ Lh = l == 0 ? mg.c16 : nullptr;
-        const int* __restrict__ Lnb = L.nb;
-        T* __restrict__ Lo = L.o;
-        const int M = *L.cnt, cap = L.cap;
-#pragma unroll 2
-        for (int i = t0; i < M; i += ns) {
-          const T ti = __ldcg(Lt + i);
-          T s = 0;
-#pragma unroll
-          for (int f = 0; f < 6; ++f) s += mg_coef(Lc, Lh, f * cap + i) * (ti - __ldcg(Lt + Lnb[f * cap + i]));
-          const T bi = __ldcg(Lb + i);
-          const T o2 = ti + w1 * Lidg[i] * (bi - s);
-          Lo[i] = o2;
-          if (l == 0) acc += bi * o2;
-        }
-      }
-    }
-    if (l == 0) block_add((double)acc, ru);
-  }
-  return 0;
-}
-
-enum { A_SUMF = 0, A_BB = 1, A_RU0 = 2, A_RR0 = 3, A_DU0 = 4, A_RU = 5, A_RR = 7, A_DU = 9, A_SUMX = 11 };
-
-// u = M^{-1} b with M = Jacobi (one level) or one multigrid V-cycle; adds (b,u) to *ru.
-template <typename T>
-__device__ __forceinline__ bool precond(const CGVec<T>& v, const MGP<T>& mg, const CGCtl& c, int M, T* b,
-                                        double* ru) {
-  if (mg.nlev > 1) {
-    CGFuse<T> off{};
-    double rr;
-    return mg_vcycle(mg, c, b, off, ru, &rr) == 0;
-  }
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-  double acc = 0;
-  for (int i = tid; i < M; i += nth) {
-    const T bi = __ldcg(b + i);
-    const T u = bi * v.idg[i];
-    v.u[i] = u;
-    acc += (double)bi * (double)u;
-  }
-  block_add(acc, ru);
-  return true;
-}
-
-// Preconditioned conjugate gradients, Chronopoulos-Gear arrangement (the recurrence
-// s = A p replaces the second matrix product of textbook CG):
-//   A: x += a p, r -= a s, rr = (r,r)                 | barrier
-//   u = M^{-1} r, gamma = (r,u)                       | barrier
-//   B: w = A u, p = u + b p, s = w + b s, delta=(w,u) | barrier
-//   b = gamma/gamma_old, a = gamma/(delta - b gamma/a_old)
-// With the multigrid preconditioner, A is folded into the first sweep of the V-cycle and
-// the residual alternates between two buffers (the sweep reads the old one at the
-// neighbours while it writes the new one).
-// Initial guess of a band solve, x0 = a + cb b + cc c over the band (b, c may be null), from
-// earlier solutions kept on the full grid; the solution is also written to hist (if set).
-template <typename T> struct CGGuess {
-  const T* a;
-  const T* b;
-  const T* c;
-  T cb, cc;
-  T* hist;
-};
-
-template <typename T, typename Rhs>
-__global__ void __launch_bounds__(1024, 1) k_cg(const int* __restrict__ idx, const int* __restrict__ count,
-                                                CGVec<T> v, T* __restrict__ wfull, Rhs rhs, CGCtl c, MGP<T> mg,
-                                                CGGuess<T> gs) {
-  const int M = *count;
-  if (M == 0) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      *c.iters = 0;
-      *c.resid = 0.0;
-    }
-    return;
-  }
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-  // one band component: the plain mean; several: the mean of each (Sec. 2.1 per component)
-  const int C = c.ncomp ? *c.ncomp : 1;
-  __shared__ double csh[kCompShared];
-  CompAcc cacc{csh, c.csum, C};
-  if (C > 1) cacc.begin();
-  double s = 0;
-  for (int i = tid; i < M; i += nth) {
-    const int p = idx[i];
-    T x0 = gs.a[p];
-    if (gs.b) x0 += gs.cb * gs.b[p];
-    if (gs.c) x0 += gs.cc * gs.c[p];
-    v.x[i] = x0;
-    const double f = rhs(p);
-    v.r1[i] = (T)f;             // f kept for the residual pass
-    if (C > 1) cacc.add(c.comp[i], (double)(T)f);
-    else s += f;
-  }
-  if (C > 1) cacc.end();
-  else block_add(s, c.acc + A_SUMF);
-  if (!grid_sync(c)) return;
-  const double meanf = *(volatile double*)(c.acc + A_SUMF) / M;
-  double bb = 0, rr = 0;
-  for (int i = tid; i < M; i += nth) {
-    double mf = meanf;
-    if (C > 1) {
-      const int ci = c.comp[i];
-      mf = __ldcg(c.csum + ci) / c.csize[ci];
-    }
-    const double b = (double)__ldcg(v.r1 + i) - mf;
-    const T r = (T)(b - (double)band_apply(v, v.x, i));
-    v.r[i] = r;
-    bb += b * b;
-    rr += (double)r * (double)r;
-  }
-  block_add(bb, c.acc + A_BB);
-  block_add(rr, c.acc + A_RR0);
-  if (!grid_sync(c)) return;
-  bb = *(volatile double*)(c.acc + A_BB);
-  rr = *(volatile double*)(c.acc + A_RR0);
-  const double tol2 = c.rtol * c.rtol * bb;
-  bool conv = (bb == 0.0) || (rr <= tol2);
-  double gamma = 0, delta = 0, alpha = 0;
-  if (!conv) {
-    if (!precond(v, mg, c, M, v.r, c.acc + A_RU0)) return;
-    if (!grid_sync(c)) return;
-    gamma = *(volatile double*)(c.acc + A_RU0);
-    double du = 0;
-    for (int i = tid; i < M; i += nth) {
-      const T w = band_apply(v, v.u, i);
-      const T u = __ldcg(v.u + i);
-      v.p[i] = u;
-      v.q[i] = w;
-      du += (double)w * (double)u;
-    }
-    block_add(du, c.acc + A_DU0);
-    if (!grid_sync(c)) return;
-    delta = *(volatile double*)(c.acc + A_DU0);
-    if (!(delta > 0.0)) conv = true;
-    alpha = conv ? 0.0 : gamma / delta;
-  }
-  const bool fuse = mg.nlev > 1;
-  int k = 0;
-  while (!conv && k < c.maxit) {
-    const int par = k & 1;
-    const T a = (T)alpha;
-    if (fuse) {
-      CGFuse<T> F{true, par ? v.r1 : v.r, v.x, v.p, v.q, a, c.acc + A_RR + par, tol2, c.acc + A_DU + (par ^ 1)};
-      const int st = mg_vcycle(mg, c, par ? v.r : v.r1, F, c.acc + A_RU + par, &rr);
-      if (st < 0) return;
-      ++k;
-      if (st == 1) {
-        conv = true;
-        break;
-      }
-    } else {
-      double rrn = 0;
-      {
-        T* __restrict__ X = v.x;
-        T* __restrict__ Rr = v.r;
-        const T* __restrict__ P = v.p;
-        const T* __restrict__ Q = v.q;
-#pragma unroll 4
-        for (int i = tid; i < M; i += nth) {
-          X[i] = __ldcg(X + i) + a * __ldcg(P + i);
-          const T r = __ldcg(Rr + i) - a * __ldcg(Q + i);
-          Rr[i] = r;
-          rrn += (double)r * (double)r;
-        }
-      }
-      block_add(rrn, c.acc + A_RR + par);
-      if (!grid_sync(c)) return;
-      if (blockIdx.x == 0 && threadIdx.x == 0) c.acc[A_DU + (par ^ 1)] = 0.0;
-      rr = *(volatile double*)(c.acc + A_RR + par);
-      ++k;
-      if (rr <= tol2) {
-        conv = true;
-        break;
-      }
-      if (!precond(v, mg, c, M, v.r, c.acc + A_RU + par)) return;
-    }
-    if (!grid_sync(c)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) c.acc[A_RR + par] = 0.0;
-    const double gnew = *(volatile double*)(c.acc + A_RU + par);
-    const double beta = gnew / gamma;
-    const T bt = (T)beta;
-    T dun = 0;
-    {
-      const T* __restrict__ U = v.u;
-      const T* __restrict__ Cc = v.c;
-      const int* __restrict__ Nb = v.nb;
-      T* __restrict__ P = v.p;
-      T* __restrict__ Q = v.q;
-      const int cap = v.cap;
-#pragma unroll 2
-      for (int i = tid; i < M; i += nth) {
-        const T u = __ldcg(U + i);
-        T w = 0;
-#pragma unroll
-        for (int f = 0; f < 6; ++f) w += Cc[f * cap + i] * (u - __ldcg(U + Nb[f * cap + i]));
-        P[i] = u + bt * __ldcg(P + i);
-        Q[i] = w + bt * __ldcg(Q + i);
-        dun += w * u;
-      }
-    }
-    block_add((double)dun, c.acc + A_DU + par);
-    if (!grid_sync(c)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) c.acc[A_RU + par] = 0.0;
-    delta = *(volatile double*)(c.acc + A_DU + par);
-    const double den = delta - beta * gnew / alpha;
-    if (!(den > 0.0)) break;
-    alpha = gnew / den;
-    gamma = gnew;
-  }
-  // zero-mean projection of the solution (per band component)
-  if (!grid_sync(c)) return;
-  double sx = 0;
-  if (C > 1) {
-    cacc.dst = c.csum + kCompCap;
-    cacc.begin();
-  }
-  for (int i = tid; i < M; i += nth) {
-    if (C > 1) cacc.add(c.comp[i], (double)__ldcg(v.x + i));
-    else sx += (double)__ldcg(v.x + i);
-  }
-  if (C > 1) cacc.end();
-  else block_add(sx, c.acc + A_SUMX);
-  if (!grid_sync(c)) return;
-  const T mx = (T)(*(volatile double*)(c.acc + A_SUMX) / M);
-  for (int i = tid; i < M; i += nth) {
-    const int p = idx[i];
-    T mi = mx;
-    if (C > 1) {
-      const int ci = c.comp[i];
-      mi = (T)(__ldcg(c.csum + kCompCap + ci) / c.csize[ci]);
-    }
-    const T w = __ldcg(v.x + i) - mi;
-    wfull[p] = w;
-    if (gs.hist) gs.hist[p] = w;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *c.iters = k;
-    *c.resid = bb > 0 ? sqrt(rr / bb) : 0.0;
-    if (!conv) atomicCAS(c.status, 0, 5);
-    atomicAdd(c.work, (unsigned long long)k * (unsigned long long)M);
-  }
-}
-
-// <w, f>: sum over the band (the nonlocal energy term).
-template <typename T, typename Rhs>
-__global__ void k_band_dot(const int* __restrict__ idx, const int* __restrict__ count, const T* __restrict__ w,
-                           Rhs rhs, double* dst) {
-  const int M = *count;
-  double s = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-    const int p = idx[i];
-    s += (double)w[p] * rhs(p);
-  }
-  block_add(s, dst);
 }
 
 }  // namespace etd

@@ -21,9 +21,10 @@ struct Error : public std::runtime_error {
   } while (0)
 
 // Tile options of a plan (0 = the default choice): pass-A z-planes per CTA, pass-B pencil
-// blocks per CTA, and direct pass-A loads/stores instead of tensor-copy staging.
+// blocks per CTA, and direct pass-A loads/stores instead of tensor-copy staging; shared: the
+// plan runs beside others (a batch), so its band solves leave SMs to them.
 struct TileOpt {
-  int zb = 0, kb = 0, direct = 0;
+  int zb = 0, kb = 0, direct = 0, shared = 0;
 };
 
 class PlanBase {

@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <vector>
+#include "bandcg.cuh"
 #include "kernels.cuh"
 #include "krylov.cuh"
 #include "ops.cuh"
@@ -51,6 +52,7 @@ template <typename T> class Stepper : public PlanBase {
     tune_zb_ = t.zb;
     tune_kb_ = t.kb;
     tune_direct_ = t.direct;
+    shared_gpu_ = t.shared != 0;
     try {
       init();
     } catch (...) {
@@ -118,12 +120,12 @@ template <typename T> class Stepper : public PlanBase {
     band_dirty_ = true;
     cg_setup(Ge);
     ETD_CUDA(cudaMemsetAsync(xe, 0, sizeof(T) * g_.n, st_));
-    cg_solve(RhsGF<T>{Ge, U}, xe);
+    cg_solve(rhs_gf(Ge, U), xe);
     ETD_CUDA(cudaMemsetAsync(scal_ + S_GRAD, 0, sizeof(double) * 5, st_));
     double init[3] = {0.0, 1e300, -1e300};
     ETD_CUDA(cudaMemcpyAsync(scal_ + S_MAXB, init, sizeof(init), cudaMemcpyHostToDevice, st_));
     k_energy_terms<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, Ge, U, ph, scal_);
-    k_band_dot<T><<<nsm_ * 4, 256, 0, st_>>>(idx_, count_, xe, RhsGF<T>{Ge, U}, scal_ + S_NONLOC);
+    k_band_dot<T><<<nsm_ * 4, 256, 0, st_>>>(idx_, count_, xe, rhs_gf(Ge, U), scal_ + S_NONLOC);
     ETD_CUDA(cudaGetLastError());
     ETD_CUDA(cudaStreamSynchronize(st_));
     double sc[S_COUNT];
@@ -184,7 +186,7 @@ template <typename T> class Stepper : public PlanBase {
     cg_setup(Ge);
     // the solution is defined on the band only
     k_zero_off_band<<<grid_for(g_.n), 256, 0, st_>>>(g_.n, mask_, (void*)xe, (int)sizeof(T));
-    cg_solve(RhsField<T>{static_cast<const T*>(f)}, xe);
+    cg_solve(Rhs<T>{RHS_FIELD, static_cast<const T*>(f), nullptr, nullptr, 0.0, ub_}, xe);
     int it = 0;
     double rs = 0;
     ETD_CUDA(cudaMemcpyAsync(&it, cg_iters_, sizeof(int), cudaMemcpyDeviceToHost, st_));
@@ -223,7 +225,7 @@ template <typename T> class Stepper : public PlanBase {
       ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
       launch_reduce(1, U, Ge, scal_ + S_MASS);
       ETD_CUDA(cudaMemsetAsync(w_, 0, sizeof(T) * g_.n, st_));
-      cg_solve(RhsGU<T>{Ge, U, P_.ubar}, w_);
+      cg_solve(rhs_gu(Ge, U), w_);
       k_r2_coupled<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, phi, static_cast<const T*>(phio_), U, w_, scal_,
                                                         hvol_, out);
     } else if (which == 3) {
@@ -234,7 +236,7 @@ template <typename T> class Stepper : public PlanBase {
       ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
       launch_reduce(2, U, Ge, scal_ + S_MASS);
       ETD_CUDA(cudaMemsetAsync(w_, 0, sizeof(T) * g_.n, st_));
-      cg_solve(RhsGF<T>{Ge, U}, w_);
+      cg_solve(rhs_gf(Ge, U), w_);
       k_r2_fixed<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, Ge, mask_, U, w_, scal_, hvol_, out);
       fixed_ready_ = false;
     } else {
@@ -311,11 +313,9 @@ template <typename T> class Stepper : public PlanBase {
     if (const char* e = std::getenv("ETD_WAIT_TRIES")) wait_tries_ = std::atoll(e);
     // shape of the band solve's multigrid cycle (tuning; every choice is a symmetric V-cycle,
     // so the preconditioned CG converges to the same tolerance): ETD_MG_LEVELS caps the levels,
-    // ETD_MG_GRID_CELLS is the full-grid size from which a level runs grid-wide (else on one
-    // block), ETD_MG_NU the smoothing sweeps per side (1 or 2), ETD_MG_CSWEEPS the Jacobi sweeps
-    // on the coarsest level (even)
+    // ETD_MG_NU the smoothing sweeps per side (1 or 2), ETD_MG_CSWEEPS the Jacobi sweeps on the
+    // coarsest level (even)
     if (const char* e = std::getenv("ETD_MG_LEVELS")) mg_maxlev_ = std::max(1, std::min(kMGMax, std::atoi(e)));
-    if (const char* e = std::getenv("ETD_MG_GRID_CELLS")) mg_grid_cells_ = std::max(1LL, std::atoll(e));
     if (const char* e = std::getenv("ETD_MG_NU")) mg_nu_ = std::atoi(e) == 1 ? 1 : 2;
     if (const char* e = std::getenv("ETD_MG_CSWEEPS")) mg_csweeps_ = std::max(2, std::atoi(e) / 2 * 2);
 
@@ -331,13 +331,25 @@ template <typename T> class Stepper : public PlanBase {
     sS_ = alloc<C>(g_.nhat);
     sSu_ = alloc<C>(g_.nhat);
     T** reals[] = {&phiA_, &phiB_, &phit_, &lap_, &gx_, &gy_, &gz_, &rr_, &wm_, &r2_, &ut_, &G_, &w_,
-                   &cg_.x, &cg_.r, &cg_.r1, &cg_.u, &cg_.p, &cg_.q, &cg_.idg};
+                   &cg_.x, &cg_.r, &cg_.p, &cg_.q};
     for (T** r : reals) *r = alloc<T>(g_.n);
     for (T** r : reals) ETD_CUDA(cudaMemset(*r, 0, sizeof(T) * g_.n));
     cg_.cap = (int)g_.n;
     cg_.c = alloc<T>(6 * (size_t)g_.n);
     cg_.nb = alloc<int>(6 * (size_t)g_.n);
     cg_.c16 = sizeof(T) == 4 ? alloc<__half>(6 * (size_t)g_.n) : nullptr;
+    if constexpr (sizeof(T) == 4) cg_.c32 = cg_.c;
+    else cg_.c32 = alloc<float>(6 * (size_t)g_.n);
+    {
+      // couplings are sums of g / h^2 with g of order one: a power of two near the smallest h^2
+      const double hm = std::min(std::min(g_.hx, g_.hy), g_.dim == 2 ? g_.hx : g_.hz);
+      cg_.csc = sizeof(T) == 4 ? (T)1 : (T)std::ldexp(1.0, 2 * std::ilogb(hm));
+    }
+    float** fl[] = {&cg_.b, &cg_.e, &cg_.o, &cg_.t, &cg_.idg};
+    for (float** f : fl) {
+      *f = alloc<float>(g_.n);
+      ETD_CUDA(cudaMemset(*f, 0, sizeof(float) * g_.n));
+    }
     bmap_ = alloc<int>(g_.n);
     cc_parent_ = alloc<int>(g_.n);
     cc_cid_ = alloc<int>(g_.n);
@@ -352,6 +364,7 @@ template <typename T> class Stepper : public PlanBase {
       ETD_CUDA(cudaMemset(h, 0, sizeof(T) * g_.n));
     }
     init_multigrid();
+    cg_prepare();
     mask_ = alloc<unsigned char>(g_.n);
     idx_ = alloc<int>(g_.n);
     idx_old_ = alloc<int>(g_.n);
@@ -363,7 +376,8 @@ template <typename T> class Stepper : public PlanBase {
     ETD_CUDA(cudaMemset(count_old_, 0, sizeof(int)));
     scal_ = alloc<double>(S_COUNT);
     ETD_CUDA(cudaMemset(scal_, 0, sizeof(double) * S_COUNT));
-    acc_ = alloc<double>(16);
+    cg_part_ = alloc<double>(A_SLOTS * kCgMaxBlocks);
+    cg_lay_ = alloc<CGLayout>(2);
     bar_ = alloc<unsigned>(2);
     status_ = alloc<int>(1);
     flag_ = alloc<int>(1);
@@ -709,7 +723,7 @@ template <typename T> class Stepper : public PlanBase {
   // Narrow band of phi: mask, ascending index list, count (device).  The previous list
   // is kept in idx_old_ so the solution can be cleared on nodes that left the band.
   void compute_band(const T* phi) {
-    cg_grid_ = 0;  // a new band: the solve's grid is the default until a frozen band sizes it
+    cg_engine_ = cg_blocks_ = 0;  // a new band: of unknown size until a frozen band is counted
     std::swap(idx_, idx_old_);
     std::swap(count_, count_old_);
     if (g_.n % 4 == 0 && (reinterpret_cast<uintptr_t>(phi) & 15) == 0) {
@@ -738,6 +752,7 @@ template <typename T> class Stepper : public PlanBase {
     CGVec<T> v = cg_;
     timed(ETD_K_BAND, 0.0, [&] { k_cg_setup<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, mask_, bmap_, G, v); });
     mg_setup();
+    cg_make_layout(kCgCluster, cg_sms());
     label_components();
     ETD_CUDA(cudaGetLastError());
   }
@@ -811,11 +826,13 @@ template <typename T> class Stepper : public PlanBase {
     return gs;
   }
 
-  template <typename Rhs> void cg_solve(Rhs rhs, T* x, CGGuess<T> gs = CGGuess<T>{}, double rtol = 0.0) {
+  Rhs<T> rhs_gu(const T* G, const T* u) const { return Rhs<T>{RHS_GU, nullptr, G, u, P_.ubar, ub_}; }
+  Rhs<T> rhs_gf(const T* G, const T* u) const { return Rhs<T>{RHS_GF, nullptr, G, u, P_.ubar, ub_}; }
+
+  void cg_solve(Rhs<T> rhs, T* x, CGGuess<T> gs = CGGuess<T>{}, double rtol = 0.0) {
     if (!gs.a) gs.a = x;
-    CGVec<T> v = cg_;
-    CGCtl c;
-    c.acc = acc_;
+    CGCtl2 q;
+    CGCtl& c = q.c;
     c.bar = bar_;
     c.status = status_;
     c.iters = cg_iters_;
@@ -828,25 +845,108 @@ template <typename T> class Stepper : public PlanBase {
     c.comp = cc_comp_;
     c.csize = csize_;
     c.csum = csum_;
-    ETD_CUDA(cudaMemsetAsync(csum_, 0, sizeof(double) * 2 * kCompCap, st_));
-    ETD_CUDA(cudaMemsetAsync(acc_, 0, sizeof(double) * 16, st_));
-    ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
-    auto k = k_cg<T, Rhs>;
-    int per = 0;
-    ETD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 1024, 0));
-    if (per < 1) throw Error(ETD_ECUDA, "band CG kernel cannot be resident");
-    const int grid = cg_grid_ > 0 ? cg_grid_ : nsm_;
+    q.part = cg_part_;
+    q.other = cg_lay_;
+    CGVec<T> v = cg_;
     const int* idx = idx_;
-    const int* cnt = count_;
     T* wfull = x;
-    MGP<T> mg = mgp();
-    void* args[] = {&idx, &cnt, &v, &wfull, &rhs, &c, &mg, &gs};
-    timed(ETD_K_CG, 0.0, [&] { ETD_CUDA(cudaLaunchCooperativeKernel((const void*)k, grid, 1024, args, 0, st_)); });
+    MGP mg = mgp();
+    // A frozen band's level counts are known: one engine.  Otherwise the band size is on the
+    // device only; grids small enough for the cluster engine launch both, and the one whose
+    // layout is not asked for returns at once (3 us, against 50 to 200 us for the solve).
+    int engine = cg_engine_;
+    if (engine == 0 && (!cluster_ok_ || g_.n > kCgClusterGrid)) engine = 2;
+    timed(ETD_K_CG, 0.0, [&] {
+      if (engine != 2) {
+        q.sel = engine == 0 ? 1 : 0;
+        q.lay = cg_lay_;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at[1];
+        cluster_config(cfg, at, cg_blocks_ > 0 ? cg_blocks_ : kCgCluster);
+        ETD_CUDA(cudaLaunchKernelEx(&cfg, k_cg<T, true>, idx, v, wfull, rhs, q, mg, gs));
+      }
+      if (engine != 1) {
+        q.sel = engine == 0 ? 2 : 0;
+        q.lay = cg_lay_ + 1;
+        ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
+        const int grid = cg_blocks_ > 0 ? cg_blocks_ : cg_sms();
+        void* args[] = {&idx, &v, &wfull, &rhs, &q, &mg, &gs};
+        ETD_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg<T, false>, grid, kCgThreads, args, grid_smem(), st_));
+      }
+    });
+  }
+
+  // Shared memory of the grid engine: where the finest matrix cannot fit (52 B a node over the
+  // blocks; bands of unknown size taken as 6% of the grid), less of it, so that L1 has the rest.
+  int grid_smem() const {
+    const double M = cg_blocks_ > 0 ? (double)fixed_count_ : 0.06 * (double)g_.n;
+    return M / (cg_blocks_ > 0 ? cg_blocks_ : cg_sms()) * 52.0 > 100.0 * 1024 ? kCgSmemBig : kCgSmem;
+  }
+  int cg_sms() const { return std::min(nsm_, kCgMaxBlocks); }
+  // Shared-memory layouts of the current band for both engines (device).
+  void cg_make_layout(int clK, int gridK) {
+    CGCounts c{};
+    for (int l = 0; l < mg_nlev_; ++l) c.cnt[l] = l == 0 ? count_ : lv_[l].cnt;
+    timed(ETD_K_BAND, 0.0, [&] { k_cg_layout<<<1, 64, 0, st_>>>(c, mg_nlev_, (int)sizeof(T), clK, gridK,
+                                                                  grid_smem(), cg_lay_); });
+    ETD_CUDA(cudaGetLastError());
+  }
+
+  void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int K) {
+    cfg.gridDim = dim3(K);
+    cfg.blockDim = dim3(kCgThreads);
+    cfg.dynamicSmemBytes = kCgSmem;
+    cfg.stream = st_;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = K;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+
+  // Shared memory and cluster size of the band solve's kernels; whether the device takes them.
+  void cg_prepare() {
+    auto kc = k_cg<T, true>;
+    auto kg = k_cg<T, false>;
+    ETD_CUDA(cudaFuncSetAttribute(kg, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem));
+    ETD_CUDA(cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem));
+    int per = 0;
+    ETD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kg, kCgThreads, kCgSmem));
+    if (per < 1) throw Error(ETD_ECUDA, "band CG kernel cannot be resident");
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    cluster_config(cfg, at, kCgCluster);
+    int ncl = 0;
+    if (cudaFuncSetAttribute(kc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&ncl, kc, &cfg) != cudaSuccess || ncl < 1) {
+      cudaGetLastError();
+      cluster_ok_ = false;
+    }
+  }
+
+  // Engine and blocks of the solves on a frozen band of known level counts.
+  void cg_choose(const int* cnt) {
+    const int M = cnt[0];
+    const int share = shared_gpu_ ? 4 : 1;
+    CGLayout y{};
+    for (int l = 0; l < mg_nlev_; ++l) y.cnt[l] = cnt[l];
+    int K = 4;
+    for (;; K *= 2) {
+      cg_layout(y, mg_nlev_, K, (int)sizeof(T), true, kCgSmem);
+      if (K == kCgCluster || (y.bytes <= kCgSmem && M <= K * kCgPerCluster * share)) break;
+    }
+    if (cluster_ok_ && y.bytes <= kCgSmem) {
+      cg_engine_ = 1;
+      cg_blocks_ = K;
+    } else {
+      cg_engine_ = 2;
+      cg_blocks_ = std::max(1, std::min(cg_sms(), (M + kCgPerBlock * share - 1) / (kCgPerBlock * share)));
+    }
+    cg_make_layout(cg_engine_ == 1 ? cg_blocks_ : kCgCluster, cg_engine_ == 2 ? cg_blocks_ : cg_sms());
   }
 
   // Level l coarsens the grid 2x per axis l times (z only in 3D) while every coarsened
-  // extent stays >= 4; levels whose full grid has >= 2^15 cells run on the whole GPU in the
-  // V-cycle, smaller ones on one block.  The cycle is V(2,2) with a degree-2 Chebyshev pair of
+  // extent stays >= 4.  The cycle is V(2,2) with a degree-2 Chebyshev pair of
   // Jacobi weights, the coarse-grid correction over-corrected by 1.9 (piecewise-constant
   // aggregation under-estimates it) and 2 sweeps on the coarsest level.
   void init_multigrid() {
@@ -854,10 +954,6 @@ template <typename T> class Stepper : public PlanBase {
     L0.ext = Ext{g_.nx, g_.ny, g_.nz};
     L0.cap = (int)g_.n;
     L0.agg = alloc<int>(g_.n);
-    L0.e = alloc<T>(g_.n);
-    L0.t = alloc<T>(g_.n);
-    ETD_CUDA(cudaMemset(L0.e, 0, sizeof(T) * g_.n));
-    ETD_CUDA(cudaMemset(L0.t, 0, sizeof(T) * g_.n));
     mg_nlev_ = 1;
     const bool is3d = g_.nz > 1;
     while (mg_nlev_ < mg_maxlev_) {
@@ -874,20 +970,18 @@ template <typename T> class Stepper : public PlanBase {
       L.map = alloc<int>(L.cap);
       L.bcount = alloc<int>(L.nblk);
       L.mark = alloc<unsigned char>(L.cap);
-      L.c = alloc<T>(6 * (size_t)L.cap);
+      L.c = alloc<float>(6 * (size_t)L.cap);
       L.nb = alloc<int>(6 * (size_t)L.cap);
-      L.idg = alloc<T>(L.cap);
+      L.idg = alloc<float>(L.cap);
       L.agg = alloc<int>(L.cap);
       L.child = alloc<int>(8 * (size_t)L.cap);
-      L.b = alloc<T>(L.cap);
-      L.e = alloc<T>(L.cap);
-      L.o = alloc<T>(L.cap);
-      L.t = alloc<T>(L.cap);
+      L.b = alloc<float>(L.cap);
+      L.e = alloc<float>(L.cap);
+      L.o = alloc<float>(L.cap);
+      L.t = alloc<float>(L.cap);
       ETD_CUDA(cudaMemset(L.cnt, 0, sizeof(int)));
       ++mg_nlev_;
     }
-    mg_gl_ = 1;
-    while (mg_gl_ < mg_nlev_ && lv_[mg_gl_].cap >= mg_grid_cells_) ++mg_gl_;
   }
 
   // Coarse levels for the current band (level 0 = idx_, count_, mask_, bmap_, cg_).  Levels
@@ -903,7 +997,7 @@ template <typename T> class Stepper : public PlanBase {
       const int* fcnt = l == 1 ? count_ : F.cnt;
       const unsigned char* fmark = l == 1 ? mask_ : F.mark;
       const int* fmap = l == 1 ? bmap_ : F.map;
-      const T* fc = l == 1 ? cg_.c : F.c;
+      const float* fc = l == 1 ? cg_.c32 : F.c;
       int* fagg = lv_[l - 1].agg;
       timed(ETD_K_BAND, 0.0, [&] {
         ETD_CUDA(cudaMemsetAsync(L.mark, 0, L.cap, st_));
@@ -919,19 +1013,19 @@ template <typename T> class Stepper : public PlanBase {
           k_band_scatter<<<L.nblk, kCompactBlock, 0, st_>>>(L.cap, L.mark, L.bcount, L.list, L.map);
         }
         k_mg_parent<<<nsm_ * 4, 256, 0, st_>>>(flist, fcnt, F.ext, is3d, L.ext, L.map, fagg);
-        k_mg_coarse<T><<<nsm_ * 4, 256, 0, st_>>>(L.list, L.cnt, L.ext, is3d, fmark, fmap, F.ext, fc,
+        k_mg_coarse<<<nsm_ * 4, 256, 0, st_>>>(L.list, L.cnt, L.ext, is3d, fmark, fmap, F.ext, fc,
                                                   F.cap, L.map, L.c, L.nb, L.idg, L.child, L.cap);
       });
       ETD_CUDA(cudaGetLastError());
     }
     if (l < mg_nlev_) {
-      MGSetTail<T> a{};
+      MGSetTail a{};
       a.first = l;
       a.nlev = mg_nlev_;
       a.is3d = is3d;
       for (int k = 0; k < mg_nlev_; ++k) {
         const HostLevel& H = lv_[k];
-        MGSetLevel<T>& S = a.L[k];
+        MGSetLevel& S = a.L[k];
         S.e = H.ext;
         S.cap = H.cap;
         S.agg = H.agg;
@@ -940,7 +1034,7 @@ template <typename T> class Stepper : public PlanBase {
           S.list = idx_;
           S.map = bmap_;
           S.mark = mask_;
-          S.c = cg_.c;
+          S.c = cg_.c32;
           S.nb = cg_.nb;
           S.idg = cg_.idg;
           S.child = nullptr;
@@ -955,15 +1049,14 @@ template <typename T> class Stepper : public PlanBase {
           S.child = H.child;
         }
       }
-      timed(ETD_K_BAND, 0.0, [&] { k_mg_setup_tail<T><<<1, 1024, 0, st_>>>(a); });
+      timed(ETD_K_BAND, 0.0, [&] { k_mg_setup_tail<<<1, 1024, 0, st_>>>(a); });
       ETD_CUDA(cudaGetLastError());
     }
   }
 
-  MGP<T> mgp() const {
-    MGP<T> m{};
+  MGP mgp() const {
+    MGP m{};
     m.nlev = mg_nlev_;
-    m.gl = mg_gl_;
     m.csweeps = mg_csweeps_;
     m.nu = mg_nu_;
     // degree-2 Chebyshev weights for D^-1 A on [lmax / 4, lmax], lmax = 2 (Gershgorin bound
@@ -971,36 +1064,36 @@ template <typename T> class Stepper : public PlanBase {
     {
       const double lmax = 2.0, lmin = lmax / 4.0, cth = 0.5 * (lmax + lmin), rad = 0.5 * (lmax - lmin);
       const double cq = std::sqrt(0.5);
-      m.w1 = (T)(1.0 / (cth + rad * cq));
-      m.w2 = (T)(1.0 / (cth - rad * cq));
+      m.w1 = (float)(1.0 / (cth + rad * cq));
+      m.w2 = (float)(1.0 / (cth - rad * cq));
     }
-    m.alpha = (T)1.9;
+    m.alpha = 1.9f;
     m.c16 = cg_.c16;
     for (int l = 0; l < mg_nlev_; ++l) {
       const HostLevel& H = lv_[l];
-      MGL<T>& L = m.L[l];
+      MGL& L = m.L[l];
       L.cap = H.cap;
       L.agg = H.agg;
-      L.e = H.e;
-      L.t = H.t;
       if (l == 0) {
         L.cnt = count_;
-        L.list = idx_;
-        L.c = cg_.c;
+        L.c = cg_.c32;
         L.nb = cg_.nb;
         L.idg = cg_.idg;
         L.child = nullptr;
-        L.b = cg_.r;
-        L.o = cg_.u;
+        L.b = cg_.b;
+        L.e = cg_.e;
+        L.o = cg_.o;
+        L.t = cg_.t;
       } else {
         L.cnt = H.cnt;
-        L.list = H.list;
         L.c = H.c;
         L.nb = H.nb;
         L.idg = H.idg;
         L.child = H.child;
         L.b = H.b;
+        L.e = H.e;
         L.o = H.o;
+        L.t = H.t;
       }
     }
     return m;
@@ -1134,7 +1227,7 @@ template <typename T> class Stepper : public PlanBase {
       launch_reduce(1, u, G_, scal_ + S_MASS);
       fwd(ProMul<T>{G_, u}, I_[0]);
       join_side_stream();
-      cg_solve(RhsGU<T>{G_, u, P_.ubar}, w_, next_guess(false, rk2), rk2 ? P_.cg_rtol_pred : 0.0);
+      cg_solve(rhs_gu(G_, u), w_, next_guess(false, rk2), rk2 ? P_.cg_rtol_pred : 0.0);
       timed(ETD_K_POINTWISE, 0.0, [&] {  // bytes from the band-node counter
         k_r2_coupled_band<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, nxt, cur, u, w_, scal_, hvol_, r2_,
                                                          cg_work_ + 1);
@@ -1145,7 +1238,7 @@ template <typename T> class Stepper : public PlanBase {
       if (rk2) {
         ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
         inv(I_[0], EpiRecoverMass<T>{ut_, G_, u, mc_.delta, ub_, scal_ + S_MASS});
-        cg_solve(RhsGU<T>{G_, ut_, P_.ubar}, w_, next_guess(true, rk2));
+        cg_solve(rhs_gu(G_, ut_), w_, next_guess(true, rk2));
         timed(ETD_K_POINTWISE, 0.0, [&] {
           k_r2_coupled_band<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, nxt, cur, ut_, w_, scal_, hvol_, r2_,
                                                            cg_work_ + 1);
@@ -1174,13 +1267,14 @@ template <typename T> class Stepper : public PlanBase {
     launch_grid(k_gloc<T>, g_.n, (const T*)phiA_, G_);
     band_for_solve(phiA_, G_);
     fixed_ready_ = true;
-    // the frozen band's size sets the band solve's grid: about 2048 nodes per block of 1024
-    // threads, so that small bands leave SMs to concurrent work (one read, once per membrane)
-    int cnt = 0;
-    ETD_CUDA(cudaMemcpyAsync(&cnt, count_, sizeof(int), cudaMemcpyDeviceToHost, st_));
+    // the frozen band's level counts choose the band solve's engine and blocks (one read, once
+    // per membrane)
+    int cnt[kMGMax] = {};
+    for (int l = 0; l < mg_nlev_; ++l)
+      ETD_CUDA(cudaMemcpyAsync(cnt + l, l == 0 ? count_ : lv_[l].cnt, sizeof(int), cudaMemcpyDeviceToHost, st_));
     ETD_CUDA(cudaStreamSynchronize(st_));
-    fixed_count_ = cnt;
-    cg_grid_ = std::max(1, std::min(nsm_, (cnt + 2047) / 2048));
+    fixed_count_ = cnt[0];
+    cg_choose(cnt);
     band_dirty_ = false;
     return true;
   }
@@ -1191,7 +1285,7 @@ template <typename T> class Stepper : public PlanBase {
     for (int n = 0; n < nsteps; ++n) {
       ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
       launch_reduce(2, u, G_, scal_ + S_MASS);
-      cg_solve(RhsGF<T>{G_, u}, w_, next_guess(false, rk2), rk2 ? P_.cg_rtol_pred : 0.0);
+      cg_solve(rhs_gf(G_, u), w_, next_guess(false, rk2), rk2 ? P_.cg_rtol_pred : 0.0);
       k_r2_fixed<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, G_, mask_, u, w_, scal_, hvol_, r2_);
       fwd(ProMul<T>{G_, u}, I_[0]);
       fwd(ProLoad<T>{r2_}, I_[1]);
@@ -1201,7 +1295,7 @@ template <typename T> class Stepper : public PlanBase {
         inv(I_[0], EpiRecover<T>{ut_, G_, u, mc_.delta});
         ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
         launch_reduce(2, ut_, G_, scal_ + S_MASS);
-        cg_solve(RhsGF<T>{G_, ut_}, w_, next_guess(true, rk2));
+        cg_solve(rhs_gf(G_, ut_), w_, next_guess(true, rk2));
         k_r2_fixed<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, G_, mask_, ut_, w_, scal_, hvol_, r2_);
         fwd(ProLoad<T>{r2_}, I_[0]);
         OpUCorr<T> ucorr{1, sSu_, sk_};
@@ -1258,7 +1352,6 @@ template <typename T> class Stepper : public PlanBase {
   void lanczos(int j0, int j1) {
     KrylovOp<T> op = kop();
     CGCtl c{};
-    c.acc = kacc_;
     c.bar = bar_;
     c.status = status_;
     c.budget = wait_budget_;
@@ -1267,7 +1360,7 @@ template <typename T> class Stepper : public PlanBase {
     int per = 0;
     ETD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 1024, 0));
     if (per < 1) throw Error(ETD_ECUDA, "Lanczos kernel cannot be resident");
-    const int grid = cg_grid_ > 0 ? cg_grid_ : nsm_;
+    const int grid = std::max(1, std::min(nsm_, (fixed_count_ + 2047) / 2048));
     const int* cnt = count_;
     T* V = kV_;
     int ld = kld_;
@@ -1352,7 +1445,7 @@ template <typename T> class Stepper : public PlanBase {
       if (nl) {
         ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
         launch_reduce(2, u, G_, scal_ + S_MASS);
-        cg_solve(RhsGF<T>{G_, u}, w_, next_guess(false, rk2), rk2 ? P_.cg_rtol_pred : 0.0);
+        cg_solve(rhs_gf(G_, u), w_, next_guess(false, rk2), rk2 ? P_.cg_rtol_pred : 0.0);
       }
       timed(ETD_K_POINTWISE, M * (11.0 * sizeof(T) + 32.0), [&] {
         k_sec2_first<T><<<nb, 256, 0, st_>>>(idx_, count_, mc_, op, ksg_, u, w_, scal_, hvol_, kR0_, kb_);
@@ -1366,7 +1459,7 @@ template <typename T> class Stepper : public PlanBase {
       if (nl) {
         ETD_CUDA(cudaMemsetAsync(scal_ + S_MASS, 0, sizeof(double), st_));
         launch_reduce(2, ut_, G_, scal_ + S_MASS);
-        cg_solve(RhsGF<T>{G_, ut_}, w_, next_guess(true, rk2));
+        cg_solve(rhs_gf(G_, ut_), w_, next_guess(true, rk2));
       }
       timed(ETD_K_POINTWISE, M * (5.0 * sizeof(T) + 4.0), [&] {
         k_sec2_second<T><<<nb, 256, 0, st_>>>(idx_, count_, mc_, ksg_, ut_, w_, scal_, hvol_, kR0_, kb_);
@@ -1500,7 +1593,14 @@ template <typename T> class Stepper : public PlanBase {
   int nsm_ = 1;
   int tune_zb_ = 0, tune_kb_ = 0;           // requested pass-A z-planes / pass-B pencil blocks (0: default)
   int tune_direct_ = 0;                      // 1: direct pass-A loads/stores (no tensor-copy staging)
-  int cg_grid_ = 0;                          // blocks of the band solve (0: one per SM)
+  // band solve: blocks, nodes per block of the grid engine, and the grid size up to which a band
+  // of unknown size may fit the cluster engine
+  static constexpr int kCgCluster = 16, kCgPerBlock = sizeof(T) == 4 ? 1024 : 512, kCgPerCluster = sizeof(T) == 4 ? 256 : 64;
+  static constexpr long long kCgClusterGrid = 1LL << 19;
+  int cg_engine_ = 0, cg_blocks_ = 0;        // frozen band: engine (1 cluster, 2 grid) and blocks; 0: unknown
+  bool cluster_ok_ = true;
+  bool shared_gpu_ = false;                  // other plans run beside this one (a batch): fewer, fuller blocks
+  CGLayout* cg_lay_ = nullptr;               // [0] cluster, [1] grid (device)
   long long wait_budget_ = 4000000000LL;   // grid barrier: clock cycles before ETD_ETIMEOUT
   long long wait_tries_ = 1LL << 22;       // pass-A tensor copy: mbarrier polls before ETD_ETIMEOUT
   size_t smemA_ = 0, smemB1_ = 0;
@@ -1527,19 +1627,18 @@ template <typename T> class Stepper : public PlanBase {
     int cap = 0, nblk = 0;
     int *cnt = nullptr, *list = nullptr, *map = nullptr, *bcount = nullptr;
     unsigned char* mark = nullptr;
-    T *c = nullptr, *idg = nullptr, *b = nullptr, *e = nullptr, *o = nullptr, *t = nullptr;
+    float *c = nullptr, *idg = nullptr, *b = nullptr, *e = nullptr, *o = nullptr, *t = nullptr;
     int *nb = nullptr, *agg = nullptr, *child = nullptr;
   };
   HostLevel lv_[kMGMax];
-  int mg_nlev_ = 1, mg_gl_ = 1;
+  int mg_nlev_ = 1;
   int mg_maxlev_ = kMGMax, mg_nu_ = 2, mg_csweeps_ = 2;
-  long long mg_grid_cells_ = 1LL << 15;
   int *idx_ = nullptr, *idx_old_ = nullptr, *bcount_ = nullptr, *count_ = nullptr, *count_old_ = nullptr;
   int nblk_ = 0;
   T* tab_ = nullptr;
   T* tabu_ = nullptr;
   C *twx_ = nullptr, *twy_ = nullptr, *twz_ = nullptr;
-  double *scal_ = nullptr, *acc_ = nullptr, *cg_resid_ = nullptr;
+  double *scal_ = nullptr, *cg_part_ = nullptr, *cg_resid_ = nullptr;
   unsigned* bar_ = nullptr;
   int *status_ = nullptr, *flag_ = nullptr, *cg_iters_ = nullptr;
   bool a0_set_ = false, fixed_ready_ = false, band_dirty_ = false, w_reset_ = true;
