@@ -56,11 +56,12 @@ etd_status scratch_address(int dev, void** out) {
 
 bool pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
-// w_N^e = exp(-2 pi i e / N) written into the scratch area on every call.
-template <typename C> __global__ void k_twiddles(C* tw, int n) {
+// w_N^e = exp(-2 pi i e / N) (team: in the team order of the long axes) written into the scratch
+// area on every call.
+template <typename C> __global__ void k_twiddles(C* tw, int n, bool team) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     double s, c;
-    sincospi(2.0 * e / n, &s, &c);
+    sincospi(2.0 * (team ? etd::team_table(n, e) : e) / n, &s, &c);
     tw[e].x = (decltype(tw[e].x))c;
     tw[e].y = (decltype(tw[e].y))(-s);
   }
@@ -100,9 +101,9 @@ etd_status run(int dim, const int* n, const void* field, void* half, cudaStream_
   C* twx = reinterpret_cast<C*>(scratch + inter);
   C* twy = reinterpret_cast<C*>(scratch + inter + align256(sizeof(C) * nx));
   C* twz = reinterpret_cast<C*>(scratch + inter + align256(sizeof(C) * nx) + align256(sizeof(C) * ny));
-  k_twiddles<C><<<4, 256, 0, st>>>(twx, nx);
-  k_twiddles<C><<<4, 256, 0, st>>>(twy, ny);
-  k_twiddles<C><<<4, 256, 0, st>>>(twz, nz);
+  k_twiddles<C><<<4, 256, 0, st>>>(twx, nx, true);
+  k_twiddles<C><<<4, 256, 0, st>>>(twy, ny, false);
+  k_twiddles<C><<<4, 256, 0, st>>>(twz, nz, true);
 
   auto ka = etd::passA_fwd<T, etd::ProLoad<T>>;
   auto kb = etd::passB<T, etd::OpToStd<T>>;

@@ -87,6 +87,9 @@ struct Geo {
 #define ETD_ZB32 4
 #endif
 
+// log2 of a power of two.
+__device__ __forceinline__ int log2_of(int n) { return 31 - __clz(n); }
+
 // Shared-memory padding: one spare slot every 16 complex elements (bank spreading).
 __host__ __device__ __forceinline__ int pad16(int k) { return k + (k >> 4); }
 
@@ -307,7 +310,9 @@ template <typename C, int N, bool INV> __device__ __forceinline__ void dftN(C* v
 
 // Team FFT of length N = R * S on S lanes (lane rank t) holding R values each, R = min(N, 16).
 // Lane t holds element t + S r in v[r] on entry and on exit, in both directions.  Forward:
-// an R-point DFT over r in registers, the twiddle w_N^(t k1), one exchange through the team's
+// an R-point DFT over r in registers, the twiddle w_N^(t k1) from the team's table
+// tw[k1 S + t] (the S lanes read consecutive entries: one L1 line, where w_N^e at e = t k1 spread
+// them over up to 16; 256^3 FP32: see team_table), one exchange through the team's
 // shared-memory scratch (pitch R + 1: conflict-free both ways), then R/S DFTs of length S
 // over the former lane index; element k1 + R k2 with k1 = t + S h lands in v[h + (R/S) k2].
 // The inverse (unnormalised) is the forward transform of the conjugate, conjugated.  scr
@@ -323,7 +328,7 @@ __device__ __forceinline__ void team_fft(C (&v)[R], int t, C* scr, const C* __re
   dftN<C, R, false>(v);
   if (S > 1) {
 #pragma unroll
-    for (int k1 = 1; k1 < R; ++k1) v[k1] = cmul(v[k1], ldg_c(&tw[t * k1]));
+    for (int k1 = 1; k1 < R; ++k1) v[k1] = cmul(v[k1], ldg_c(&tw[k1 * S + t]));
     __syncwarp();
     if (act) {
 #pragma unroll
@@ -347,6 +352,10 @@ __device__ __forceinline__ void team_fft(C (&v)[R], int t, C* scr, const C* __re
   }
 }
 
+// Exponent of entry e of an axis' team table, w_N^(t k1) at e = k1 S + t (the tables of x and z;
+// y, whose twiddles are uniform over a block, keeps w_N^e).
+__host__ __device__ __forceinline__ int team_table(int n, int e) { return (e % team_S(n)) * (e / team_S(n)); }
+
 // Wavenumber bookkeeping of one spectral element.
 struct Wave {
   int kx, ky, kz;   // raw spectral indices (kx < Nx/2+1)
@@ -361,18 +370,22 @@ __device__ __forceinline__ void fold(int i, int n, int& f, int& s) {
   s = (i < h) ? i : (i == h ? 0 : i - n);
 }
 
-__device__ __forceinline__ Wave make_wave(const Geo& g, int kx, int ky, int kz) {
-  Wave w;
+// The x and y part of a row's elements, and one element of it (N = Nz at compile time).
+__device__ __forceinline__ Wave make_wave_row(const Geo& g, int kx, int ky) {
+  Wave w{};
   w.kx = kx;
   w.ky = ky;
-  w.kz = kz;
   fold(kx, g.nx, w.fx, w.sx);
   fold(ky, g.ny, w.fy, w.sy);
-  fold(kz, g.nz, w.fz, w.sz);
-  w.m = w.fx * w.fx + w.fy * w.fy + w.fz * w.fz;
+  w.m = w.fx * w.fx + w.fy * w.fy;
   return w;
 }
-
+template <int N> __device__ __forceinline__ Wave make_wave_z(Wave w, int kz) {
+  w.kz = kz;
+  fold(kz, N, w.fz, w.sz);
+  w.m += w.fz * w.fz;
+  return w;
+}
 
 // Inverse pass-A epilogues: epi(i, v) stores output i.  One with kSums also adds terms to
 // the partial sums of a row pair (Epi::Part, live only while the pair is stored), which
@@ -397,17 +410,19 @@ template <typename T, typename Pro, int R, int S>
 __device__ __forceinline__ void passA_rows_fwd(const Geo& g, const Pro& pro, typename Cplx<T>::type* tile, int rs,
                                                int z0, int n1, const typename Cplx<T>::type* __restrict__ twx) {
   using C = typename Cplx<T>::type;
+  constexpr int N = R * S, half = N / 2;
   const int t = threadIdx.x & (S - 1);
   const int team = threadIdx.x / S, nteams = blockDim.x / S;
-  const int ncrows = (g.ZB * g.Y2) >> 1;
-  const int half = g.nx >> 1;
-  for (int base = 0; base < ncrows; base += nteams) {
+  const int ncrows = (g.ZB * g.Y2) >> 1, ly = log2_of(g.Y2);
+  // a warp whose teams all lack a row pair skips the round: its lanes would run the transform
+  // on zeros (128^3 FP64, 4 of 16 warps with rows: 220 -> 105 us a launch, FP64-pipe bound)
+  for (int base = 0; base < ncrows && base + (int)(threadIdx.x & ~31u) / S < ncrows; base += nteams) {
     const int q = base + team;
     const bool ok = q < ncrows;
     C v[R];
-    const int r0 = 2 * q, r1 = r0 + 1;
-    const long long i0 = ((long long)(z0 + r0 / g.Y2) * g.ny + n1 + g.Y1 * (r0 % g.Y2)) * g.nx;
-    const long long i1 = ((long long)(z0 + r1 / g.Y2) * g.ny + n1 + g.Y1 * (r1 % g.Y2)) * g.nx;
+    const int r0 = 2 * q;   // Y2 is even: both rows of a pair are in one plane
+    const long long i0 = ((long long)(z0 + (r0 >> ly)) * g.ny + n1 + g.Y1 * (r0 & (g.Y2 - 1))) * N;
+    const long long i1 = i0 + (long long)g.Y1 * N;
 #pragma unroll
     for (int j = 0; j < R; ++j) {
       const int x = t + S * j;
@@ -449,7 +464,7 @@ __device__ __forceinline__ void passA_cols_fwd(const Geo& g, const typename Cplx
   using C = typename Cplx<T>::type;
   const int ncols = g.ZB * g.nxh;
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
-    const int zz = col % g.ZB, kx = col / g.ZB;
+    const int zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
     C v[Y > 1 ? Y : 1];
 #pragma unroll
     for (int j = 0; j < Y; ++j) v[j] = tile[(zz * Y + j) * rs + pad16(kx)];
@@ -530,7 +545,7 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
   const int nmain = ncols < nt ? ncols : nt, ntail = ncols - nmain;
   C v[Y > 1 ? Y : 1];
   if (t < ntail) {
-    const int col = nmain + t, zz = col % g.ZB, kx = col / g.ZB;
+    const int col = nmain + t, zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
 #pragma unroll
     for (int j = 0; j < Y; ++j) v[j] = tile[(zz * Y + j) * rs + pad16(kx)];
     dftN<C, Y, false>(v);
@@ -538,7 +553,7 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
     for (int k2 = 0; k2 < Y; ++k2) side[t * Y + k2] = (n1 && k2) ? cmul(v[k2], ldg_c(&twy[n1 * k2])) : v[k2];
   }
   const bool mine = t < nmain;
-  const int zz = t % g.ZB, kx = t / g.ZB;
+  const int zz = t & (g.ZB - 1), kx = t >> log2_of(g.ZB);
   if (mine) {
 #pragma unroll
     for (int j = 0; j < Y; ++j) v[j] = tile[(zz * Y + j) * rs + pad16(kx)];
@@ -555,7 +570,7 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
   }
   if (t < ntail * Y) {
     const int tcol = nmain + t / Y, tk2 = t % Y;
-    stg[(tk2 * g.nxh + tcol / g.ZB) * g.ZB + tcol % g.ZB] = side[t];
+    stg[(tk2 * g.nxh + (tcol >> log2_of(g.ZB))) * g.ZB + (tcol & (g.ZB - 1))] = side[t];
   }
 }
 
@@ -612,7 +627,7 @@ __device__ __forceinline__ void passA_cols_inv(const Geo& g, typename Cplx<T>::t
   using C = typename Cplx<T>::type;
   const int ncols = g.ZB * g.nxh;
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
-    const int zz = col % g.ZB, kx = col / g.ZB;
+    const int zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
     C v[Y > 1 ? Y : 1];
 #pragma unroll
     for (int k2 = 0; k2 < Y; ++k2) {
@@ -638,7 +653,7 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
   const int nmain = ncols < nt ? ncols : nt, ntail = ncols - nmain;
   C v[Y > 1 ? Y : 1];
   const bool mine = t < nmain;
-  const int zz = t % g.ZB, kx = t / g.ZB;
+  const int zz = t & (g.ZB - 1), kx = t >> log2_of(g.ZB);
   if (mine) {
 #pragma unroll
     for (int k2 = 0; k2 < Y; ++k2) v[k2] = stg[(k2 * g.nxh + kx) * g.ZB + zz];
@@ -646,7 +661,7 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
   const bool tl = t < ntail * Y;
   const int tcol = nmain + t / Y, tk2 = t % Y;
   C xt = C{0, 0};
-  if (tl) xt = stg[(tk2 * g.nxh + tcol / g.ZB) * g.ZB + tcol % g.ZB];
+  if (tl) xt = stg[(tk2 * g.nxh + (tcol >> log2_of(g.ZB))) * g.ZB + (tcol & (g.ZB - 1))];
   __syncthreads();
   if (mine) {
     if (n1) {
@@ -660,11 +675,11 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
   if (ntail > 0) {
     if (tl) {
       if (n1) xt = cmulc(xt, ldg_c(&twy[n1 * tk2]));
-      tile[((tcol % g.ZB) * Y + tk2) * rs + pad16(tcol / g.ZB)] = xt;
+      tile[((tcol & (g.ZB - 1)) * Y + tk2) * rs + pad16(tcol >> log2_of(g.ZB))] = xt;
     }
     __syncthreads();
     if (t < ntail) {
-      const int col = nmain + t, z2 = col % g.ZB, k = col / g.ZB;
+      const int col = nmain + t, z2 = col & (g.ZB - 1), k = col >> log2_of(g.ZB);
 #pragma unroll
       for (int k2 = 0; k2 < Y; ++k2) v[k2] = tile[(z2 * Y + k2) * rs + pad16(k)];
       dftN<C, Y, true>(v);
@@ -679,14 +694,16 @@ __device__ __forceinline__ void passA_rows_inv(const Geo& g, const Epi& epi, typ
                                                int z0, int n1, const typename Cplx<T>::type* __restrict__ twx,
                                                typename Epi::Acc& acc) {
   using C = typename Cplx<T>::type;
+  constexpr int N = R * S, half = N / 2;
   const int t = threadIdx.x & (S - 1);
   const int team = threadIdx.x / S, nteams = blockDim.x / S;
-  const int ncrows = (g.ZB * g.Y2) >> 1;
-  const int N = g.nx, half = g.nx >> 1;
-  for (int base = 0; base < ncrows; base += nteams) {
+  const int ncrows = (g.ZB * g.Y2) >> 1, ly = log2_of(g.Y2);
+  for (int base = 0; base < ncrows && base + (int)(threadIdx.x & ~31u) / S < ncrows; base += nteams) {
     const int q = base + team;
     const bool ok = q < ncrows;
-    const int r0 = 2 * q, r1 = r0 + 1;
+    const int r0 = 2 * q;
+    const long long i0 = ((long long)(z0 + (r0 >> ly)) * g.ny + n1 + g.Y1 * (r0 & (g.Y2 - 1))) * N;
+    const long long i1 = i0 + (long long)g.Y1 * N;
     C* ra = tile + (ok ? r0 : 0) * rs;
     const C* rb = ra + rs;
     C v[R];
@@ -712,16 +729,12 @@ __device__ __forceinline__ void passA_rows_inv(const Geo& g, const Epi& epi, typ
       v[r] = C{A.x - B.y, A.y + B.x};
     }
     if (ok && Epi::kPrefetch) {
-      const long long p0 = ((long long)(z0 + r0 / g.Y2) * g.ny + n1 + g.Y1 * (r0 % g.Y2)) * g.nx;
-      const long long p1 = ((long long)(z0 + r1 / g.Y2) * g.ny + n1 + g.Y1 * (r1 % g.Y2)) * g.nx;
-      const int nl = N >= 32 ? N / 32 : 1;
-      for (int q = t; q < 2 * nl; q += S) epi.prefetch((q < nl ? p0 : p1) + 32 * (q % nl));
+      constexpr int nl = N >= 32 ? N / 32 : 1;
+      for (int q = t; q < 2 * nl; q += S) epi.prefetch((q < nl ? i0 : i1) + 32 * (q % nl));
     }
     // the pair's rows, now held in registers, serve as the exchange scratch
     team_fft<C, R, S, true>(v, t, ra, twx, ok);
     if (ok) {
-      const long long i0 = ((long long)(z0 + r0 / g.Y2) * g.ny + n1 + g.Y1 * (r0 % g.Y2)) * g.nx;
-      const long long i1 = ((long long)(z0 + r1 / g.Y2) * g.ny + n1 + g.Y1 * (r1 % g.Y2)) * g.nx;
       typename Epi::Part part{};
 #pragma unroll
       for (int j = 0; j < R; ++j) {
@@ -876,6 +889,9 @@ __device__ __forceinline__ void passB_rows(const Geo& g, const Op& op, int kx0, 
   const int t = threadIdx.x & (S - 1);
   const int team = threadIdx.x / S, nteams = blockDim.x / S;
   const int nrows = kbn * g.Y1;
+  constexpr int N = R * S;
+  // a warp whose teams all lack a row takes part in the column stages and barriers only
+  const int wteam = (int)(threadIdx.x & ~31u) / S;
   // spectra kept in registers across the outputs
   C base[RPT][R];
   int rowid[RPT];
@@ -883,6 +899,7 @@ __device__ __forceinline__ void passB_rows(const Geo& g, const Op& op, int kx0, 
   for (int rr = 0; rr < RPT; ++rr) {
     const int row = team + rr * nteams;
     rowid[rr] = row;
+    if (wteam + rr * nteams >= nrows) continue;
     const bool ok = row < nrows;
     C* r0 = tile0 + (ok ? row : 0) * rs;
     C* r1 = tile1 + (ok ? row : 0) * rs;
@@ -899,11 +916,12 @@ __device__ __forceinline__ void passB_rows(const Geo& g, const Op& op, int kx0, 
     }
     if (ok) {
       const int kxl = row / g.Y1, k1 = row - kxl * g.Y1;
+      const Wave wr = make_wave_row(g, kx0 + kxl, k2 + g.Y2 * k1);
 #pragma unroll
       for (int k = 0; k < R; ++k) {
         const int kz = t + S * k;
-        const Wave w = make_wave(g, kx0 + kxl, k2 + g.Y2 * k1, kz);
-        const int e = row * g.nz + kz;
+        const Wave w = make_wave_z<N>(wr, kz);
+        const int e = row * N + kz;
         op.combine(e, cb + e, w, s0[k], s1[k]);
         base[rr][k] = s0[k];
       }
@@ -921,14 +939,13 @@ __device__ __forceinline__ void passB_rows(const Geo& g, const Op& op, int kx0, 
 #pragma unroll
     for (int rr = 0; rr < RPT; ++rr) {
       const int row = rowid[rr];
+      if (wteam + rr * nteams >= nrows) continue;
       const bool ok = row < nrows;
       C v[R];
       const int kxl = ok ? row / g.Y1 : 0, k1 = ok ? row - kxl * g.Y1 : 0;
+      const Wave wr = make_wave_row(g, kx0 + kxl, k2 + g.Y2 * k1);
 #pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const int kz = t + S * k;
-        v[k] = ok ? op.out(o, base[rr][k], make_wave(g, kx0 + kxl, k2 + g.Y2 * k1, kz)) : C{0, 0};
-      }
+      for (int k = 0; k < R; ++k) v[k] = ok ? op.out(o, base[rr][k], make_wave_z<N>(wr, t + S * k)) : C{0, 0};
       C* r0 = tb + (ok ? row : 0) * rs;
       team_fft<C, R, S, true>(v, t, r0, twz, ok);
       __syncwarp();

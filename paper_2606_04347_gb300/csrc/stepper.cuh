@@ -389,10 +389,11 @@ template <typename T> class Stepper : public PlanBase {
     ETD_CUDA(cudaMemset(cg_iters_, 0, sizeof(int)));
     ETD_CUDA(cudaMemset(cg_resid_, 0, sizeof(double)));
 
-    // twiddle tables w_N^e = exp(-2 pi i e / N) and the phi-function table, built in FP64
-    twx_ = upload_twiddles(nx);
-    twy_ = upload_twiddles(ny);
-    twz_ = upload_twiddles(nz);
+    // twiddle tables w_N^e = exp(-2 pi i e / N) (x, z: in team order) and the phi-function table,
+    // built in FP64
+    twx_ = upload_twiddles(nx, true);
+    twy_ = upload_twiddles(ny, false);
+    twz_ = upload_twiddles(nz, true);
     if constexpr (sizeof(T) == 4) {
       if (P_.model == ETD_MODEL_COUPLED && g_.nz > 1) init_df(optin);
     }
@@ -437,11 +438,11 @@ template <typename T> class Stepper : public PlanBase {
     ETD_CUDA(cudaDeviceSynchronize());
   }
 
-  template <typename E = T> typename Cplx<E>::type* upload_twiddles(int n) {
+  template <typename E = T> typename Cplx<E>::type* upload_twiddles(int n, bool team) {
     using CE = typename Cplx<E>::type;
     std::vector<CE> t(n);
     for (int e = 0; e < n; ++e) {
-      const long double a = 2.0L * 3.14159265358979323846264338327950288L * e / n;
+      const long double a = 2.0L * 3.14159265358979323846264338327950288L * (team ? team_table(n, e) : e) / n;
       t[e].x = E((double)cosl(a));
       t[e].y = E((double)(-sinl(a)));
     }
@@ -462,9 +463,9 @@ template <typename T> class Stepper : public PlanBase {
     sphi_d_ = alloc<dcomplex>(g_.nhat);
     Id_ = alloc<dcomplex>(g_.nhat);
     philo_ = alloc<T>(g_.n);
-    twx_d_ = upload_twiddles<dfloat>(g_.nx);
-    twy_d_ = upload_twiddles<dfloat>(g_.ny);
-    twz_d_ = upload_twiddles<dfloat>(g_.nz);
+    twx_d_ = upload_twiddles<dfloat>(g_.nx, true);
+    twy_d_ = upload_twiddles<dfloat>(g_.ny, false);
+    twz_d_ = upload_twiddles<dfloat>(g_.nz, true);
     dfphi_ = true;
   }
 
