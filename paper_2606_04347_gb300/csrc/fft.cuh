@@ -125,7 +125,10 @@ __host__ __device__ __forceinline__ int pitch_b(int nz) {
 //           4 (8-byte complex) or 2 (16-byte complex);
 //   pass B: KB consecutive kx pencil blocks of Y1 x Nz per CTA.  A team of S lanes takes one
 //           row (two in 2D), so KB Y1 is at most the block's rows; kb_req > 0 asks for KB, else
-//           1 in 3D (the most CTAs) and as many as the block holds in 2D.
+//           in 3D as many as give four warps a row each (an SM sub-partition without one idles
+//           its pipes in the row stages: 128^3 FP64 KB 1 -> 2 869 -> 595 us a predictor launch,
+//           64^3 FP32 KB 1 -> 4 39 -> 21 us) while 140 CTAs are left, and as many as the block
+//           holds in 2D.
 inline int passb_max_rows(int nz) {
   const int rpt = team_R(nz) >= 8 ? 1 : 2;
   return (ETD_PASSB_THREADS / team_S(nz)) * rpt;
@@ -145,7 +148,9 @@ inline bool choose_tiles(Geo& g, size_t csize, size_t& smemA, size_t& smemB1, in
   if (kb_req > 0) {
     g.KB = kb_req;
   } else if (g.nz > 1) {
+    const int ctas = g.nxh * g.Y2;
     g.KB = 1;
+    while (2 * g.KB <= kbmax && 2 * g.KB * g.Y1 * team_S(g.nz) <= 128 && ctas / (2 * g.KB) >= 140) g.KB *= 2;
   } else {
     g.KB = 512 / g.Y1;
   }
