@@ -1132,7 +1132,12 @@ template <typename T> class Stepper : public PlanBase {
   // R1 parts at (phi, u): rr_ = R1 without the Laplacian term, wm_ = W'(phi) - A1 phi.
   void phi_terms(const T* phi, const T* u) {
     timed(ETD_K_POINTWISE, (g_.nz > 1 ? 8 : 7) * fld(), [&] {
-      k_r1<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, phi, lap_, gx_, gy_, gz_, u, scal_, hvol_, rr_, wm_);
+      constexpr int V = 16 / sizeof(T);
+      const bool al = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(phi)) & 15) == 0 && g_.n % V == 0;
+      if (al)
+        k_r1<T, V><<<grid_for(g_.n / V), 256, 0, st_>>>(g_, mc_, phi, lap_, gx_, gy_, gz_, u, scal_, hvol_, rr_, wm_);
+      else
+        k_r1<T, 1><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, phi, lap_, gx_, gy_, gz_, u, scal_, hvol_, rr_, wm_);
     });
     ETD_CUDA(cudaGetLastError());
   }
