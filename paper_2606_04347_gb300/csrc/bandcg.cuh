@@ -6,7 +6,7 @@
 // them and, on this part, every FP64 instruction (an SM issues 2 FP64 operations per clock: one
 // warp instruction holds its pipe for 64 clocks, a block-wide FP64 shuffle reduction of 1024
 // threads takes 1.5 us).  Hence
-//   * two engines, the same arithmetic:
+//   * three engines, the same arithmetic:
 //       cluster  one thread-block cluster holds the whole solve in shared memory (matrix,
 //                vectors, all levels); neighbours are read through distributed shared memory and
 //                phases are separated by the cluster barrier (0.3 us; 0.8 us when global stores
@@ -14,6 +14,8 @@
 //       grid     up to one block per SM, vectors in global memory (L2), each block's share of the
 //                matrix cached in shared memory where it fits, a grid barrier (1.2 us) between
 //                phases;
+//       hybrid   the grid engine on clusters: the finest level(s) as there, and every cluster runs
+//                the coarser ones on a copy of its own, as the cluster engine would;
 //   * levels of at most kCgLocal nodes run in every block on its own copy in shared memory, so
 //     the small levels cost block barriers only and their result needs no broadcast;
 //   * reductions and scalars of the FP32 form are double-float (FP32 pipes), and the FP64 form's
@@ -125,20 +127,24 @@ struct MGP {
 // held whole by every block.
 struct CGLayout {
   int cnt[kMGMax];
+  int lg;              // levels below lg are spread over all blocks, [lg, lc) over each cluster
   int lc;
   int n[kMGMax];       // nodes per block of a distributed level (a multiple of 32)
   int mat[kMGMax];     // byte offset of the cached matrix (distributed: c, nb code, idg, child code;
                        // local: c, idg, nb, child), -1: read from global memory
-  int vec[kMGMax];     // byte offset of b, e, o, t (cluster engine, and local levels)
+  int vec[kMGMax];     // byte offset of b, e, o, t (levels of a cluster, and local levels)
   int cgv;             // byte offset of x, r, p, q (cluster engine)
   int c64;             // byte offset of the FP64 couplings, -1: read from global memory
   int agg;             // byte offset of the parents of level lc - 1's own nodes (16-bit), -1: global
+  int par;             // hybrid: byte offset of the parent codes of level lg - 1's own nodes
   int lchild;          // byte offset of level lc's child codes
-  int bytes;           // what the layout needs; cluster engine: more than kCgSmem means it does not fit
+  int bytes;           // what the layout needs; more than `smem`: it does not fit
 };
-// Fills y from y.cnt.  Cluster: everything has to fit; grid: matrices are cached while there is
-// room, the finest level first (it takes five of the phases).
-__host__ __device__ inline void cg_layout(CGLayout& y, int nlev, int K, int tsize, bool cluster, int smem) {
+enum { CG_GRID = 0, CG_CLUSTER = 1, CG_HYBRID = 2 };
+// Fills y from y.cnt for K blocks in clusters of KC.  Cluster: everything has to fit; hybrid: the
+// levels of the clusters have to; matrices of the grid's levels are cached while there is room,
+// the finest level first (it takes five of the phases).
+__host__ __device__ inline void cg_layout(CGLayout& y, int nlev, int K, int KC, int tsize, int mode, int smem) {
   int at = 0;
   auto take = [&at](int b) {
     const int o = at;
@@ -146,15 +152,36 @@ __host__ __device__ inline void cg_layout(CGLayout& y, int nlev, int K, int tsiz
     return o;
   };
   int lc = nlev;
-  while (lc > 1 && y.cnt[lc - 1] <= (cluster ? kCgLocal : kCgLocalGrid)) --lc;
-  y.agg = y.lchild = y.cgv = y.c64 = -1;
+  while (lc > 1 && y.cnt[lc - 1] <= (mode == CG_GRID ? kCgLocalGrid : kCgLocal)) --lc;
   // local levels that would not fit go back to the distributed ones
   for (int b = 0; lc < nlev; ++lc, b = 0) {
     for (int l = lc; l < nlev; ++l) b += 72 * y.cnt[l] + 64;
     if (b + 16 * y.cnt[lc] <= smem) break;
   }
   y.lc = lc;
-  for (int l = 0; l < lc; ++l) y.n[l] = ((y.cnt[l] + K - 1) / K + 31) & ~31;
+  y.agg = y.lchild = y.cgv = y.c64 = y.par = -1;
+  y.bytes = smem + 1;
+  int lg = mode == CG_CLUSTER ? 0 : lc;
+  if (mode == CG_HYBRID) {
+    // the first level from which a cluster holds all the rest (16 + 84 B a node, local levels and
+    // the finer level's parent codes beside them)
+    int room = smem - 8192;
+    for (int l = lc; l < nlev; ++l) room -= 72 * y.cnt[l] + 64;
+    if (lc < nlev) room -= 16 * y.cnt[lc];
+    lg = lc;
+    for (int l = lc - 1; l >= 1; --l) {
+      const int n = ((y.cnt[l] + KC - 1) / KC + 31) & ~31;
+      if (n > room / 100) break;
+      room -= 100 * n;
+      if (4 * ((y.cnt[l - 1] + K - 1) / K + 31) <= room) lg = l;
+    }
+    if (lg >= lc || lg >= nlev - 1) return;   // nothing for the clusters to do
+  }
+  y.lg = lg;
+  for (int l = 0; l < lc; ++l) {
+    const int k = l < lg ? K : KC;
+    y.n[l] = ((y.cnt[l] + k - 1) / k + 31) & ~31;
+  }
   if (lc < nlev) {
     for (int l = lc; l < nlev; ++l) {
       const int m = y.cnt[l];
@@ -163,46 +190,53 @@ __host__ __device__ inline void cg_layout(CGLayout& y, int nlev, int K, int tsiz
     }
     y.lchild = take(32 * y.cnt[lc]);
   }
-  for (int l = 0; l < lc; ++l) {
+  for (int l = lg; l < lc; ++l) {
+    const int n = y.n[l];
+    if (n > smem / 52) return;   // more than a block holds (and no overflow below)
+    y.vec[l] = take(16 * n);
+    if (l == 0) y.cgv = take(4 * tsize * n);
+    y.mat[l] = take((l > 0 ? 84 : 52) * n);
+    if (l == 0 && tsize == 8) y.c64 = take(48 * n);
+  }
+  if (mode == CG_HYBRID) y.par = take(4 * y.n[lg - 1]);
+  if (lc < nlev && lc > lg && mode != CG_GRID) y.agg = take(2 * y.n[lc - 1]);
+  for (int l = 0; l < lg; ++l) {
     const int n = y.n[l], per = l > 0 ? 84 : 52;
     y.mat[l] = y.vec[l] = -1;
-    if (n > smem / 52) {   // more than a block holds (and no overflow below)
-      if (cluster) {
-        y.bytes = smem + 1;
-        return;
-      }
-      continue;
-    }
-    if (cluster) {
-      y.vec[l] = take(16 * n);
-      if (l == 0) y.cgv = take(4 * tsize * n);
-    }
-    if (cluster || at + per * n <= smem) y.mat[l] = take(per * n);
-    if (l == 0 && tsize == 8 && (cluster || at + 48 * n <= smem)) y.c64 = take(48 * n);
+    if (n > smem / 52) continue;
+    if (at + per * n <= smem) y.mat[l] = take(per * n);
+    if (l == 0 && tsize == 8 && at + 48 * n <= smem) y.c64 = take(48 * n);
   }
-  if (lc < nlev && (cluster || at + 2 * y.n[lc - 1] <= smem)) y.agg = take(2 * y.n[lc - 1]);
+  if (mode == CG_GRID && lc < nlev && at + 2 * y.n[lc - 1] <= smem) y.agg = take(2 * y.n[lc - 1]);
   y.bytes = at;
 }
 
 struct CGCtl2 {
   CGCtl c;
-  const CGLayout* lay; // this engine's layout
-  const CGLayout* other; // sel = 2: the cluster engine's layout
-  double* part;        // per-block partial sums of the grid engine, kCgMaxBlocks per slot
-  int sel;             // 0: run; 1: run if the cluster layout fits; 2: run if it does not
+  const CGLayout* lay;   // this engine's layout
+  const CGLayout* other; // sel & 2: the layout of the engine that goes first
+  double* part;          // per-block partial sums (grid, hybrid), kCgMaxBlocks per slot
+  int sel;               // 1: run only if this layout fits; 2: only if the other one does not
+  int KC;                // blocks of a cluster
 };
 
-// One thread per engine: layouts for clK blocks (cluster) and gridK blocks (grid).
+// One warp per layout: [0] the cluster engine's for clK blocks, [1] the grid engine's for gridK,
+// [2] the hybrid engine's for hybK in clusters of kCgCluster.
+constexpr int kCgCluster = 16;
 struct CGCounts {
   const int* cnt[kMGMax];
 };
-static __global__ void k_cg_layout(CGCounts cs, int nlev, int tsize, int clK, int gridK, int gsmem,
+static __global__ void k_cg_layout(CGCounts cs, int nlev, int tsize, int clK, int gridK, int hybK, int gsmem,
                                    CGLayout* out) {
-  __shared__ CGLayout y[2];
+  __shared__ CGLayout y[3];
   const int e = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (l < kMGMax) y[e].cnt[l] = l < nlev ? *cs.cnt[l] : 0;
   __syncwarp();
-  if (l == 0) cg_layout(y[e], nlev, e == 0 ? clK : gridK, tsize, e == 0, e == 0 ? kCgSmem : gsmem);
+  if (l == 0) {
+    if (e == 0) cg_layout(y[e], nlev, clK, clK, tsize, CG_CLUSTER, kCgSmem);
+    if (e == 1) cg_layout(y[e], nlev, gridK, 1, tsize, CG_GRID, gsmem);
+    if (e == 2) cg_layout(y[e], nlev, hybK, kCgCluster, tsize, CG_HYBRID, kCgSmem);
+  }
   __syncwarp();
   for (int k = l; k < (int)(sizeof(CGLayout) / 4); k += 32)
     reinterpret_cast<int*>(out + e)[k] = reinterpret_cast<const int*>(&y[e])[k];
@@ -341,10 +375,11 @@ struct LevL {
   }
 };
 
-template <typename T, bool CL> struct CGShared {
+template <typename T> struct CGShared {
   using W = typename WideOf<T>::type;
   CGLayout lay;
-  LevD<CL> d[kMGMax];
+  LevD<false> dg[kMGMax];   // levels of the grid
+  LevD<true> dc[kMGMax];    // levels of a cluster
   alignas(8) W part[6];   // this block's partial sums (cluster engine)
   W ws[2][32];
   W gamma, alpha;         // written and read by one thread
@@ -386,29 +421,31 @@ template <typename Load, typename Store> __device__ __forceinline__ void nodes(i
   nodes(n, load, [] {}, store);
 }
 
-template <typename T, bool CL> struct CGSolve {
+template <typename T, int MODE> struct CGSolve {
   using W = typename WideOf<T>::type;
-  CGShared<T, CL>& S;
+  static constexpr bool CL = MODE == CG_CLUSTER;
+  CGShared<T>& S;
   const CGCtl2& q;
   const MGP& mg;
   int rank, K;
   uint32_t dyn;   // address of the dynamic shared memory
 
-  // Barrier over the blocks of the solve.  Cluster: the hardware barrier (it does not spin; a
-  // budget below zero still gives up).  Grid: the arrival counter of grid_sync; a flag per block
-  // that every block polls measured 2 to 5 us against its 1.3 us (152 blocks, the polls' traffic).
-  __device__ bool bar() const {
-    if constexpr (CL) {
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-      if (q.c.budget < 0) {
-        if (threadIdx.x == 0) atomicCAS(q.c.status, 0, 6);
-        return false;
-      }
-      return true;
-    } else {
-      return grid_sync(q.c);
+  // Barrier over a cluster: the hardware barrier (it does not spin; a budget below zero still
+  // gives up).
+  __device__ bool cbar() const {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (q.c.budget < 0) {
+      if (threadIdx.x == 0) atomicCAS(q.c.status, 0, 6);
+      return false;
     }
+    return true;
+  }
+  // Barrier over all blocks of the solve: the arrival counter of grid_sync (a flag per block that
+  // every block polls measured 2 to 5 us against its 1.3 us at 152 blocks: the polls' traffic).
+  __device__ bool bar() const {
+    if constexpr (CL) return cbar();
+    else return grid_sync(q.c);
   }
   // Block sum of v into this block's partial `slot`; warps from nact on hold zero.  The caller
   // takes a barrier before total(), and between two posts of slots of the same parity.
@@ -452,150 +489,226 @@ template <typename T, bool CL> struct CGSolve {
   // visible to every block: o = M^-1 b.  Residuals of the pre-sweeps are carried algebraically:
   // r1 = b - A e1, d = w2 D^-1 r1, e2 = e1 + d, r2 = r1 - A d; r2 is gathered into the parent
   // aggregates (the restriction of piecewise-constant P), and a level's correction is added to
-  // its children's e by the thread that computed it.  `before` runs before the first phase (the
+  // its children's e by the thread that computed it (or, where the coarser level is this block's
+  // or its cluster's own copy, by the child's).  `before` runs before the first phase (the
   // scalar warp forms the stopping test there) and S.go is looked at after the first barrier.
   // `dot` sees every own (node, o).  Returns -1 if a barrier gave up, 1 if the test stopped the
   // solve, 0 with o complete except for the barrier that the caller takes.
   template <typename Before, typename Dot> __device__ int vcycle(Before&& before, Dot&& dot) const {
     const int nlev = mg.nlev, lc = S.lay.lc, last = nlev - 1, ld = lc < last ? lc : last;
-    const float w1 = mg.w1, w2 = mg.w2, al = mg.alpha;
-    const bool two = mg.nu == 2;
+    const int lg = MODE == CG_GRID ? lc : (MODE == CG_CLUSTER ? 0 : S.lay.lg);
+    const auto gb = [&] { return bar(); };
+    const auto cb = [&] { return cbar(); };
+    const auto none = [](int, float) {};
     before();
     if (nlev == 1) {
       __syncthreads();
       if (!S.go) return 1;
-      const LevD<CL> L = S.d[0];
-      nodes(
-          L.n, [&](int s) { return L.idg(s) * L.own(V_B, s); },
-          [&](int s, float o) {
-            L.put(V_O, s, o);
-            dot(s, o);
-          });
-      return 0;
-    }
-    for (int l = 0; l < ld; ++l) {
-      const LevD<CL> L = S.d[l];
-      nodes(
-          L.n,
-          [&](int s) {
-            const float r1 = L.own(V_B, s) - lap_d(L, V_E, s, L.own(V_E, s), false);
-            return make_float2(r1, w2 * L.idg(s) * r1);
-          },
-          [&](int s, float2 r) {
-            L.put(V_O, s, r.x);
-            L.put(V_T, s, r.y);
-          });
-      if (!bar()) return -1;
-      if (l == 0 && !S.go) return 1;
-      if (two) {
+      auto jac = [&](auto L) {
         nodes(
-            L.n,
-            [&](int s) {
-              const float d = L.own(V_T, s);
-              return make_float2(L.own(V_O, s) - lap_d(L, V_T, s, d, true), L.own(V_E, s) + d);
-            },
-            [&](int s, float2 r) {
-              L.put(V_O, s, r.x);
-              L.put(V_E, s, r.y);
-            });
-        if (!bar()) return -1;
-      }
-      if (l + 1 < lc) {
-        const LevD<CL> N = S.d[l + 1];
-        nodes(
-            N.n,
-            [&](int s) {
-              const float b = child_sum(N, L, V_O, s);
-              return make_float2(b, w1 * N.idg(s) * b);
-            },
-            [&](int s, float2 r) {
-              N.put(V_B, s, r.x);
-              N.put(V_E, s, r.y);
-            });
-        if (!bar()) return -1;
-      }
-    }
-    if (lc < nlev) {
-      local_cycle();
-      // the correction of level lc to this block's nodes of level lc - 1
-      const LevD<CL> L = S.d[lc - 1];
-      const LevL C = loc(lc);
-      const int* agg = mg.L[lc - 1].agg + (size_t)rank * S.lay.n[lc - 1];
-      const int a16 = S.lay.agg;
-      nodes(
-          L.n,
-          [&](int s) {
-            const int p = a16 >= 0 ? (int)lds_h(dyn + a16 + 2 * s) : agg[s];
-            return L.own(V_E, s) + al * lds_f(C.v(V_O, p));
-          },
-          [&](int s, float e) { L.put(V_E, s, e); });
-      if (!bar()) return -1;
-    } else {
-      const LevD<CL> L = S.d[last];   // e = w1 D^-1 b is the first sweep
-      for (int k = 1; k < mg.csweeps; ++k) {
-        const int src = (k & 1) ? V_E : V_O, dst = (k & 1) ? V_O : V_E;
-        const float w = (k & 1) ? w2 : w1;
-        nodes(
-            L.n,
-            [&](int s) {
-              const float v = L.own(src, s);
-              return v + w * L.idg(s) * (L.own(V_B, s) - lap_d(L, src, s, v, true));
-            },
-            [&](int s, float v) { L.put(dst, s, v); });
-        if (!bar()) return -1;
-      }
-      push(last);
-      if (!bar()) return -1;
-    }
-    for (int l = ld - 1; l >= 0; --l) {
-      const LevD<CL> L = S.d[l];
-      const float ws = two ? w2 : w1;
-      const int out = two ? V_T : V_O;
-      nodes(
-          L.n,
-          [&](int s) {
-            const float e = L.own(V_E, s);
-            return e + ws * L.idg(s) * (L.own(V_B, s) - lap_d(L, V_E, s, e, true));
-          },
-          [&](int s, float o) {
-            L.put(out, s, o);
-            if (l == 0 && !two) dot(s, o);
-          });
-      if (two) {
-        if (!bar()) return -1;
-        nodes(
-            L.n,
-            [&](int s) {
-              const float t = L.own(V_T, s);
-              return t + w1 * L.idg(s) * (L.own(V_B, s) - lap_d(L, V_T, s, t, true));
-            },
+            L.n, [&](int s) { return L.idg(s) * L.own(V_B, s); },
             [&](int s, float o) {
               L.put(V_O, s, o);
-              if (l == 0) dot(s, o);
+              dot(s, o);
             });
+      };
+      if constexpr (CL) jac(S.dc[0]);
+      else jac(S.dg[0]);
+      return 0;
+    }
+    // down
+    if constexpr (MODE != CG_CLUSTER) {
+      for (int l = 0; l < ld && l < lg; ++l) {
+        const LevD<false> L = S.dg[l];
+        if (!sweep1(L, gb)) return -1;
+        if (l == 0 && !S.go) return 1;
+        if (!sweep2(L, gb)) return -1;
+        if (l + 1 < lg && !gather(LevD<false>(S.dg[l + 1]), L, gb)) return -1;
       }
-      if (l > 0) {
-        push(l);
+    }
+    if constexpr (MODE != CG_GRID) {
+      if constexpr (MODE == CG_HYBRID) {
+        if (!gather(LevD<true>(S.dc[lg]), LevD<false>(S.dg[lg - 1]), cb)) return -1;
+      }
+      for (int l = lg; l < ld; ++l) {
+        const LevD<true> L = S.dc[l];
+        if (!sweep1(L, cb)) return -1;
+        if (l == 0 && !S.go) return 1;
+        if (!sweep2(L, cb)) return -1;
+        if (l + 1 < lc && !gather(LevD<true>(S.dc[l + 1]), L, cb)) return -1;
+      }
+    }
+    // the coarsest levels
+    bool ok;
+    if constexpr (MODE == CG_GRID) ok = bottom(S.dg, gb);
+    else ok = bottom(S.dc, cb);
+    if (!ok) return -1;
+    // up
+    if constexpr (MODE != CG_GRID) {
+      for (int l = ld - 1; l >= lg; --l) {
+        const LevD<true> L = S.dc[l];
+        if (CL && l == 0) {
+          if (!post_sweeps(L, cb, dot)) return -1;
+          continue;
+        }
+        if (!post_sweeps(L, cb, none)) return -1;
+        if (l > lg) push(L, LevD<true>(S.dc[l - 1]));
+        if (!cbar()) return -1;
+      }
+      if constexpr (MODE == CG_HYBRID) {
+        // the cluster's correction to this block's own nodes of level lg - 1
+        const LevD<false> L = S.dg[lg - 1];
+        const LevD<true> N = S.dc[lg];
+        const uint32_t par = dyn + (uint32_t)S.lay.par;
+        const float al = mg.alpha;
+        nodes(
+            L.n, [&](int s) { return L.own(V_E, s) + al * N.nbr(V_O, lds_u(par + 4 * s)); },
+            [&](int s, float e) { L.put(V_E, s, e); });
+        if (!bar()) return -1;
+      }
+    }
+    if constexpr (MODE != CG_CLUSTER) {
+      for (int l = (lg < ld ? lg : ld) - 1; l >= 0; --l) {
+        const LevD<false> L = S.dg[l];
+        if (l == 0) {
+          if (!post_sweeps(L, gb, dot)) return -1;
+          continue;
+        }
+        if (!post_sweeps(L, gb, none)) return -1;
+        push(L, LevD<false>(S.dg[l - 1]));
         if (!bar()) return -1;
       }
     }
     return 0;
   }
 
-  // e += alpha o on the children of this block's nodes of level l (each node has one parent).
-  __device__ void push(int l) const {
-    const LevD<CL> N = S.d[l], L = S.d[l - 1];
-    for (int s = threadIdx.x; s < N.n; s += kCgThreads) {
-      const float o = mg.alpha * N.own(V_O, s);
+  // r1 = b - A e into o, d = w2 D^-1 r1 into t.
+  template <class L, class B> __device__ __forceinline__ bool sweep1(const L& A, B&& b) const {
+    const float w2 = mg.w2;
+    nodes(
+        A.n,
+        [&](int s) {
+          const float r1 = A.own(V_B, s) - lap_d(A, V_E, s, A.own(V_E, s), false);
+          return make_float2(r1, w2 * A.idg(s) * r1);
+        },
+        [&](int s, float2 r) {
+          A.put(V_O, s, r.x);
+          A.put(V_T, s, r.y);
+        });
+    return b();
+  }
+  // r2 = r1 - A d into o, e += d.
+  template <class L, class B> __device__ __forceinline__ bool sweep2(const L& A, B&& b) const {
+    if (mg.nu != 2) return true;
+    nodes(
+        A.n,
+        [&](int s) {
+          const float d = A.own(V_T, s);
+          return make_float2(A.own(V_O, s) - lap_d(A, V_T, s, d, true), A.own(V_E, s) + d);
+        },
+        [&](int s, float2 r) {
+          A.put(V_O, s, r.x);
+          A.put(V_E, s, r.y);
+        });
+    return b();
+  }
+  // The residual of level F into the right-hand side of the next level N, and its first sweep.
+  template <class N, class L, class B> __device__ __forceinline__ bool gather(const N& A, const L& F, B&& b) const {
+    const float w1 = mg.w1;
+    nodes(
+        A.n,
+        [&](int s) {
+          const float r = child_sum(A, F, V_O, s);
+          return make_float2(r, w1 * A.idg(s) * r);
+        },
+        [&](int s, float2 r) {
+          A.put(V_B, s, r.x);
+          A.put(V_E, s, r.y);
+        });
+    return b();
+  }
+  // The sweeps after the coarse-grid correction; the barrier after the last is the caller's.
+  template <class L, class B, class Dot>
+  __device__ __forceinline__ bool post_sweeps(const L& A, B&& b, Dot&& dot) const {
+    const bool two = mg.nu == 2;
+    const float ws = two ? mg.w2 : mg.w1, w1 = mg.w1;
+    const int out = two ? V_T : V_O;
+    nodes(
+        A.n,
+        [&](int s) {
+          const float e = A.own(V_E, s);
+          return e + ws * A.idg(s) * (A.own(V_B, s) - lap_d(A, V_E, s, e, true));
+        },
+        [&](int s, float o) {
+          A.put(out, s, o);
+          if (!two) dot(s, o);
+        });
+    if (!two) return true;
+    if (!b()) return false;
+    nodes(
+        A.n,
+        [&](int s) {
+          const float t = A.own(V_T, s);
+          return t + w1 * A.idg(s) * (A.own(V_B, s) - lap_d(A, V_T, s, t, true));
+        },
+        [&](int s, float o) {
+          A.put(V_O, s, o);
+          dot(s, o);
+        });
+    return true;
+  }
+  // The local levels and their correction to level lc - 1, or the sweeps of a coarsest level that
+  // is distributed and its push; ends with a barrier.
+  template <class L, class B> __device__ bool bottom(const L* d, B&& b) const {
+    const int nlev = mg.nlev, lc = S.lay.lc, last = nlev - 1;
+    if (lc < nlev) {
+      const L A = d[lc - 1];
+      local_cycle(A);
+      const LevL C = loc(lc);
+      const float al = mg.alpha;
+      const int a16 = S.lay.agg;
+      // blocks of the level's tier: the whole grid, or this cluster
+      const int tr = MODE == CG_HYBRID ? rank % q.KC : rank;
+      const int* agg = mg.L[lc - 1].agg + (size_t)tr * S.lay.n[lc - 1];
+      nodes(
+          A.n,
+          [&](int s) {
+            const int p = a16 >= 0 ? (int)lds_h(dyn + a16 + 2 * s) : agg[s];
+            return A.own(V_E, s) + al * lds_f(C.v(V_O, p));
+          },
+          [&](int s, float e) { A.put(V_E, s, e); });
+      return b();
+    }
+    const L A = d[last];   // e = w1 D^-1 b is the first sweep
+    for (int k = 1; k < mg.csweeps; ++k) {
+      const int src = (k & 1) ? V_E : V_O, dst = (k & 1) ? V_O : V_E;
+      const float w = (k & 1) ? mg.w2 : mg.w1;
+      nodes(
+          A.n,
+          [&](int s) {
+            const float v = A.own(src, s);
+            return v + w * A.idg(s) * (A.own(V_B, s) - lap_d(A, src, s, v, true));
+          },
+          [&](int s, float v) { A.put(dst, s, v); });
+      if (!b()) return false;
+    }
+    push(A, d[last - 1]);
+    return b();
+  }
+
+  // e += alpha o on the children of this block's nodes of level N (each node has one parent).
+  template <class N, class L> __device__ void push(const N& A, const L F) const {
+    for (int s = threadIdx.x; s < A.n; s += kCgThreads) {
+      const float o = mg.alpha * A.own(V_O, s);
       unsigned ch[8];
       float e[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) ch[k] = N.child(k, s);
+      for (int k = 0; k < 8; ++k) ch[k] = A.child(k, s);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) e[k] = ch[k] != ~0u ? L.nbr(V_E, ch[k]) : 0.0f;
+      for (int k = 0; k < 8; ++k) e[k] = ch[k] != ~0u ? F.nbr(V_E, ch[k]) : 0.0f;
 #pragma unroll
       for (int k = 0; k < 8; ++k)
-        if (ch[k] != ~0u) L.put_nbr(V_E, ch[k], e[k] + o);
+        if (ch[k] != ~0u) F.put_nbr(V_E, ch[k], e[k] + o);
     }
   }
 
@@ -604,12 +717,11 @@ template <typename T, bool CL> struct CGSolve {
   // take part (a named barrier), and from the first level of at most 32 nodes on one warp goes
   // alone: a phase is then a warp barrier and a few shared-memory latencies.  Ends with the
   // result o of level lc visible to the block.
-  __device__ void local_cycle() const {
+  template <class L> __device__ void local_cycle(const L& F) const {
     const int nlev = mg.nlev, lc = S.lay.lc;
     const int s = threadIdx.x, nthr = (S.lay.cnt[lc] + 31) & ~31;
     if (s < nthr) {
       const LevL N = loc(lc);
-      const LevD<CL> L = S.d[lc - 1];
       if (s < N.n) {
         const uint32_t lch = dyn + (uint32_t)S.lay.lchild + 4 * s;
         struct {
@@ -617,7 +729,7 @@ template <typename T, bool CL> struct CGSolve {
           int n;
           __device__ unsigned child(int k, int) const { return lds_u(a + 4 * k * n); }
         } codes{lch, N.n};
-        const float b = child_sum(codes, L, V_O, s);
+        const float b = child_sum(codes, F, V_O, s);
         sts_f(N.v(V_B, s), b);
         sts_f(N.v(V_E, s), mg.w1 * N.idg(s) * b);
       }
@@ -728,19 +840,20 @@ enum { A_SUMF = 0, A_BB = 1, A_RR = 2, A_RU = 3, A_DU = 4, A_SUMX = 5, A_SLOTS =
 //   o = M^{-1} b, gamma = (r,o)                                        | barrier
 //   w = A o, p = o + beta p, s = w + beta s, delta = (w,o)             | barrier
 //   beta = gamma/gamma_old, a = gamma/(delta - beta gamma/a_old)
-template <typename T, bool CL>
+template <typename T, int MODE>
 __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ idx, CGVec<T> v, T* __restrict__ wfull,
                                                       Rhs<T> rhs, CGCtl2 q, MGP mg, CGGuess<T> gs) {
   using W = typename WideOf<T>::type;
+  constexpr bool CL = MODE == CG_CLUSTER;
   extern __shared__ __align__(16) unsigned char cg_dyn[];
-  __shared__ CGShared<T, CL> S;
+  __shared__ CGShared<T> S;
   const int rank = blockIdx.x, K = gridDim.x, t0 = threadIdx.x;
   const CGCtl& c = q.c;
   if (t0 < (int)(sizeof(CGLayout) / 4)) reinterpret_cast<int*>(&S.lay)[t0] = reinterpret_cast<const int*>(q.lay)[t0];
-  const int skip = q.sel == 2 ? q.other->bytes <= kCgSmem : 0;
+  const int skip = (q.sel & 2) ? q.other->bytes <= kCgSmem : 0;
   const int st0 = *(volatile int*)c.status;   // an earlier failure (too many components, a lost copy): no solve
   __syncthreads();
-  if (skip || st0 != 0 || (q.sel == 1 && S.lay.bytes > kCgSmem)) return;
+  if (skip || st0 != 0 || ((q.sel & 1) && S.lay.bytes > kCgSmem)) return;
   const int M = S.lay.cnt[0];
   if (M == 0) {
     if (rank == 0 && t0 == 0) {
@@ -752,17 +865,20 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
   const uint32_t dyn = smem_u32(cg_dyn);
   const int na0 = S.lay.n[0], base = rank * na0;
   const int n0 = max(0, min(na0, M - base));
-  const int lc = S.lay.lc, nlev = mg.nlev;
+  const int lc = S.lay.lc, nlev = mg.nlev, lg = MODE == CG_GRID ? lc : (CL ? 0 : S.lay.lg);
+  const int crank = MODE == CG_HYBRID ? rank % q.KC : rank;   // rank in the cluster
   if (t0 < lc) {
-    const int l = t0, na = S.lay.n[l], lb = rank * na;
+    const int l = t0, na = S.lay.n[l], lb = (l < lg ? rank : crank) * na, n = max(0, min(na, S.lay.cnt[l] - lb));
     const MGL& G = mg.L[l];
-    LevD<CL>& L = S.d[l];
-    L.n = max(0, min(na, S.lay.cnt[l] - lb));
-    if constexpr (CL) {
+    if (l >= lg) {
+      LevD<true>& L = S.dc[l];
+      L.n = n;
       L.st = 4 * na;
       L.mat = dyn + (uint32_t)S.lay.mat[l];
       L.vec = dyn + (uint32_t)S.lay.vec[l];
     } else {
+      LevD<false>& L = S.dg[l];
+      L.n = n;
       L.lb = lb;
       L.c16 = nullptr;
       L.g[0] = G.b;
@@ -787,34 +903,33 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
     }
   }
   __syncthreads();
-  // Matrices into shared memory.  Codes: the address of the node's element in its level's first
-  // vector (cluster; j / na by a multiply, exact for the j < 2^32 / na of a level that fits), or j.
+  // Matrices into shared memory.  Code of node j of a level: the address of its element in the
+  // level's first vector where a cluster holds it (j / na by a multiply, exact for the
+  // j < 2^32 / na of a level that fits), else j.
+  auto code = [&](int l, int j, unsigned mul) -> unsigned {
+    if (MODE == CG_GRID || l < lg) return (unsigned)j;
+    const unsigned na = (unsigned)S.lay.n[l], r = __umulhi((unsigned)j, mul);
+    return mapa_u32(dyn + (uint32_t)S.lay.vec[l], r) + 4u * ((unsigned)j - r * na);
+  };
+  auto magic = [&](int l) { return 0xffffffffu / (unsigned)S.lay.n[l] + 1u; };
   for (int l = 0; l < lc; ++l) {
     if (S.lay.mat[l] < 0) continue;
     const MGL& G = mg.L[l];
-    const int na = S.lay.n[l], lb = rank * na, nf = l > 0 ? S.lay.n[l - 1] : 32;
-    const unsigned mul = 0xffffffffu / (unsigned)na + 1u, mulf = 0xffffffffu / (unsigned)nf + 1u;
-    const uint32_t va = dyn + (uint32_t)S.lay.vec[l], vf = l > 0 ? dyn + (uint32_t)S.lay.vec[l - 1] : 0;
+    const int na = S.lay.n[l], lb = (l < lg ? rank : crank) * na, n = max(0, min(na, S.lay.cnt[l] - lb));
+    const unsigned mul = magic(l), mulf = l > 0 ? magic(l - 1) : 0;
     unsigned char* m = cg_dyn + S.lay.mat[l];
-    auto code = [&](int j, int n, unsigned mu, uint32_t vb) -> unsigned {
-      if constexpr (CL) {
-        const unsigned r = __umulhi((unsigned)j, mu);
-        return mapa_u32(vb, r) + 4u * ((unsigned)j - r * (unsigned)n);
-      }
-      return (unsigned)j;
-    };
-    for (int s = t0; s < S.d[l].n; s += kCgThreads) {
+    for (int s = t0; s < n; s += kCgThreads) {
 #pragma unroll
       for (int f = 0; f < 6; ++f) {
         reinterpret_cast<float*>(m)[f * na + s] = G.c[f * G.cap + lb + s];
-        reinterpret_cast<unsigned*>(m + 24 * na)[f * na + s] = code(G.nb[f * G.cap + lb + s], na, mul, va);
+        reinterpret_cast<unsigned*>(m + 24 * na)[f * na + s] = code(l, G.nb[f * G.cap + lb + s], mul);
       }
       reinterpret_cast<float*>(m + 48 * na)[s] = G.idg[lb + s];
       if (l > 0) {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int ch = G.child[k * G.cap + lb + s];
-          reinterpret_cast<unsigned*>(m + 52 * na)[k * na + s] = ch < 0 ? ~0u : code(ch, nf, mulf, vf);
+          reinterpret_cast<unsigned*>(m + 52 * na)[k * na + s] = ch < 0 ? ~0u : code(l - 1, ch, mulf);
         }
       }
     }
@@ -822,6 +937,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
   for (int l = lc; l < nlev; ++l) {
     const MGL& G = mg.L[l];
     const int m = S.lay.cnt[l];
+    const unsigned mulf = magic(lc - 1);
     unsigned char* p = cg_dyn + S.lay.mat[l];
     for (int s = t0; s < m; s += kCgThreads) {
 #pragma unroll
@@ -833,24 +949,21 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int ch = G.child[k * G.cap + s];
-        if (l > lc) {
-          reinterpret_cast<unsigned short*>(p + 40 * m)[k * m + s] = ch < 0 ? 0xffff : (unsigned short)(4 * ch);
-        } else {
-          unsigned cd = (unsigned)ch;
-          if constexpr (CL) {
-            const int nf = S.lay.n[lc - 1];
-            const int r = ch < 0 ? 0 : ch / nf;
-            if (ch >= 0) cd = mapa_u32(dyn + (uint32_t)S.lay.vec[lc - 1], r) + 4u * (unsigned)(ch - r * nf);
-          }
-          reinterpret_cast<unsigned*>(cg_dyn + S.lay.lchild)[k * m + s] = cd;
-        }
+        if (l > lc) reinterpret_cast<unsigned short*>(p + 40 * m)[k * m + s] = ch < 0 ? 0xffff : (unsigned short)(4 * ch);
+        else reinterpret_cast<unsigned*>(cg_dyn + S.lay.lchild)[k * m + s] = ch < 0 ? ~0u : code(lc - 1, ch, mulf);
       }
     }
   }
   if (S.lay.agg >= 0) {
-    const int lb = rank * S.lay.n[lc - 1];
-    for (int s = t0; s < S.d[lc - 1].n; s += kCgThreads)
+    const int na = S.lay.n[lc - 1], lb = (lc - 1 < lg ? rank : crank) * na, n = max(0, min(na, S.lay.cnt[lc - 1] - lb));
+    for (int s = t0; s < n; s += kCgThreads)
       reinterpret_cast<unsigned short*>(cg_dyn + S.lay.agg)[s] = (unsigned short)mg.L[lc - 1].agg[lb + s];
+  }
+  if constexpr (MODE == CG_HYBRID) {
+    const unsigned mul = magic(lg);
+    const int lb = rank * S.lay.n[lg - 1];
+    for (int s = t0; s < S.dg[lg - 1].n; s += kCgThreads)
+      reinterpret_cast<unsigned*>(cg_dyn + S.lay.par)[s] = code(lg, mg.L[lg - 1].agg[lb + s], mul);
   }
   // x, r, p, q of the own nodes; the CG operator's couplings
   T *X = v.x + base, *R = v.r + base, *P = v.p + base, *Q = v.q + base;
@@ -875,8 +988,10 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
       csA = v.cap;
     }
   }
-  const CGSolve<T, CL> A{S, q, mg, rank, K, dyn};
-  const LevD<CL> L0 = S.d[0];
+  const CGSolve<T, MODE> A{S, q, mg, rank, K, dyn};
+  LevD<CL> L0;
+  if constexpr (CL) L0 = S.dc[0];
+  else L0 = S.dg[0];
   auto cop = [&](int f, int i) -> T {
     if constexpr (sizeof(T) == 4) return L0.c(f, i, false);
     else return cA[f * csA + i];
@@ -1108,7 +1223,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
     if (!conv) atomicCAS(c.status, 0, 5);
     atomicAdd(c.work, (unsigned long long)k * (unsigned long long)M);
   }
-  if constexpr (CL) A.bar();   // no block leaves while another still reads its shared memory
+  if constexpr (MODE != CG_GRID) A.cbar();   // no block leaves while another still reads its shared memory
 }
 
 // <w, f>: sum over the band (the nonlocal energy term).

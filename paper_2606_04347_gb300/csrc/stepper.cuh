@@ -377,7 +377,7 @@ template <typename T> class Stepper : public PlanBase {
     scal_ = alloc<double>(S_COUNT);
     ETD_CUDA(cudaMemset(scal_, 0, sizeof(double) * S_COUNT));
     cg_part_ = alloc<double>(A_SLOTS * kCgMaxBlocks);
-    cg_lay_ = alloc<CGLayout>(2);
+    cg_lay_ = alloc<CGLayout>(3);
     bar_ = alloc<unsigned>(2);
     status_ = alloc<int>(1);
     flag_ = alloc<int>(1);
@@ -753,7 +753,7 @@ template <typename T> class Stepper : public PlanBase {
     CGVec<T> v = cg_;
     timed(ETD_K_BAND, 0.0, [&] { k_cg_setup<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, mask_, bmap_, G, v); });
     mg_setup();
-    cg_make_layout(kCgCluster, cg_sms());
+    cg_make_layout();
     label_components();
     ETD_CUDA(cudaGetLastError());
   }
@@ -847,32 +847,33 @@ template <typename T> class Stepper : public PlanBase {
     c.csize = csize_;
     c.csum = csum_;
     q.part = cg_part_;
-    q.other = cg_lay_;
     CGVec<T> v = cg_;
     const int* idx = idx_;
     T* wfull = x;
     MGP mg = mgp();
     // A frozen band's level counts are known: one engine.  Otherwise the band size is on the
-    // device only; grids small enough for the cluster engine launch both, and the one whose
-    // layout is not asked for returns at once (3 us, against 50 to 200 us for the solve).
-    int engine = cg_engine_;
-    if (engine == 0 && (!cluster_ok_ || g_.n > kCgClusterGrid)) engine = 2;
+    // device only and two are launched, of which one returns at once (3 us, against 50 to 300 us
+    // for the solve): the cluster or, on larger grids, the hybrid engine where its layout fits,
+    // and the grid engine where it does not; the grid engine alone where neither can.
+    int first = cg_engine_ - 1, second = -1;
+    if (cg_engine_ == 0) {
+      first = !cluster_ok_ || g_.n > kCgHybridGrid ? CG_GRID : (g_.n > kCgClusterGrid ? CG_HYBRID : CG_CLUSTER);
+      if (first != CG_GRID) second = CG_GRID;
+    }
+    q.KC = kCgCluster;
     timed(ETD_K_CG, 0.0, [&] {
-      if (engine != 2) {
-        q.sel = engine == 0 ? 1 : 0;
-        q.lay = cg_lay_;
+      if (first != CG_CLUSTER || second >= 0) ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
+      for (int e : {first, second}) {
+        if (e < 0) continue;
+        q.sel = second < 0 ? 0 : (e == first ? 1 : 2);
+        q.lay = cg_lay_ + (e == CG_CLUSTER ? 0 : e == CG_GRID ? 1 : 2);
+        q.other = cg_lay_ + (first == CG_CLUSTER ? 0 : 2);
         cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute at[1];
-        cluster_config(cfg, at, cg_blocks_ > 0 ? cg_blocks_ : kCgCluster);
-        ETD_CUDA(cudaLaunchKernelEx(&cfg, k_cg<T, true>, idx, v, wfull, rhs, q, mg, gs));
-      }
-      if (engine != 1) {
-        q.sel = engine == 0 ? 2 : 0;
-        q.lay = cg_lay_ + 1;
-        ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
-        const int grid = cg_blocks_ > 0 ? cg_blocks_ : cg_sms();
-        void* args[] = {&idx, &v, &wfull, &rhs, &q, &mg, &gs};
-        ETD_CUDA(cudaLaunchCooperativeKernel((const void*)k_cg<T, false>, grid, kCgThreads, args, grid_smem(), st_));
+        cudaLaunchAttribute at[2];
+        cg_config(cfg, at, e, cg_blocks_ > 0 ? cg_blocks_ : cg_default_blocks(e));
+        if (e == CG_CLUSTER) ETD_CUDA(cudaLaunchKernelEx(&cfg, k_cg<T, CG_CLUSTER>, idx, v, wfull, rhs, q, mg, gs));
+        else if (e == CG_HYBRID) ETD_CUDA(cudaLaunchKernelEx(&cfg, k_cg<T, CG_HYBRID>, idx, v, wfull, rhs, q, mg, gs));
+        else ETD_CUDA(cudaLaunchKernelEx(&cfg, k_cg<T, CG_GRID>, idx, v, wfull, rhs, q, mg, gs));
       }
     });
   }
@@ -884,66 +885,96 @@ template <typename T> class Stepper : public PlanBase {
     return M / (cg_blocks_ > 0 ? cg_blocks_ : cg_sms()) * 52.0 > 100.0 * 1024 ? kCgSmemBig : kCgSmem;
   }
   int cg_sms() const { return std::min(nsm_, kCgMaxBlocks); }
-  // Shared-memory layouts of the current band for both engines (device).
-  void cg_make_layout(int clK, int gridK) {
+  int cg_default_blocks(int e) const { return e == CG_CLUSTER ? kCgCluster : e == CG_GRID ? cg_sms() : hyb_blocks_; }
+  // Shared-memory layouts of the current band for the engines (device).
+  void cg_make_layout() {
     CGCounts c{};
     for (int l = 0; l < mg_nlev_; ++l) c.cnt[l] = l == 0 ? count_ : lv_[l].cnt;
-    timed(ETD_K_BAND, 0.0, [&] { k_cg_layout<<<1, 64, 0, st_>>>(c, mg_nlev_, (int)sizeof(T), clK, gridK,
-                                                                  grid_smem(), cg_lay_); });
+    auto blocks = [&](int e) { return cg_engine_ == e + 1 ? cg_blocks_ : cg_default_blocks(e); };
+    timed(ETD_K_BAND, 0.0, [&] {
+      k_cg_layout<<<1, 96, 0, st_>>>(c, mg_nlev_, (int)sizeof(T), blocks(CG_CLUSTER), blocks(CG_GRID),
+                                     std::max(blocks(CG_HYBRID), kCgCluster), grid_smem(), cg_lay_);
+    });
     ETD_CUDA(cudaGetLastError());
   }
 
-  void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int K) {
-    cfg.gridDim = dim3(K);
+  void cg_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int e, int blocks) {
+    cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kCgThreads);
-    cfg.dynamicSmemBytes = kCgSmem;
+    cfg.dynamicSmemBytes = e == CG_GRID ? grid_smem() : kCgSmem;
     cfg.stream = st_;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = K;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 0;
+    if (e != CG_GRID) {
+      cudaLaunchAttribute& a = at[cfg.numAttrs++];
+      a.id = cudaLaunchAttributeClusterDimension;
+      a.val.clusterDim.x = e == CG_CLUSTER ? blocks : kCgCluster;
+      a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    }
+    if (e != CG_CLUSTER) {   // blocks that wait on one another across clusters: all resident
+      cudaLaunchAttribute& a = at[cfg.numAttrs++];
+      a.id = cudaLaunchAttributeCooperative;
+      a.val.cooperative = 1;
+    }
   }
 
-  // Shared memory and cluster size of the band solve's kernels; whether the device takes them.
+  // Shared memory and cluster sizes of the band solve's kernels; whether the device takes them.
   void cg_prepare() {
-    auto kc = k_cg<T, true>;
-    auto kg = k_cg<T, false>;
+    auto kc = k_cg<T, CG_CLUSTER>;
+    auto kg = k_cg<T, CG_GRID>;
+    auto kh = k_cg<T, CG_HYBRID>;
     ETD_CUDA(cudaFuncSetAttribute(kg, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem));
     ETD_CUDA(cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem));
+    ETD_CUDA(cudaFuncSetAttribute(kh, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem));
     int per = 0;
     ETD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kg, kCgThreads, kCgSmem));
     if (per < 1) throw Error(ETD_ECUDA, "band CG kernel cannot be resident");
     cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    cluster_config(cfg, at, kCgCluster);
-    int ncl = 0;
+    cudaLaunchAttribute at[2];
+    cg_config(cfg, at, CG_CLUSTER, kCgCluster);
+    int nc = 0, nh = 0;
     if (cudaFuncSetAttribute(kc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&ncl, kc, &cfg) != cudaSuccess || ncl < 1) {
+        cudaFuncSetAttribute(kh, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&nc, kc, &cfg) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&nh, kh, &cfg) != cudaSuccess || nc < 1 || nh < 1) {
       cudaGetLastError();
       cluster_ok_ = false;
     }
+    hyb_blocks_ = kCgCluster * std::max(1, std::min(nh, kCgMaxBlocks / kCgCluster));
   }
 
-  // Engine and blocks of the solves on a frozen band of known level counts.
+  // Engine and blocks of the solves on a frozen band of known level counts: a cluster if it
+  // holds the band, else the hybrid engine if a cluster holds the coarser levels, else the grid.
   void cg_choose(const int* cnt) {
-    const int M = cnt[0];
-    const int share = shared_gpu_ ? 4 : 1;
+    const int M = cnt[0], share = shared_gpu_ ? 4 : 1;
     CGLayout y{};
     for (int l = 0; l < mg_nlev_; ++l) y.cnt[l] = cnt[l];
-    int K = 4;
-    for (;; K *= 2) {
-      cg_layout(y, mg_nlev_, K, (int)sizeof(T), true, kCgSmem);
-      if (K == kCgCluster || (y.bytes <= kCgSmem && M <= K * kCgPerCluster * share)) break;
+    cg_engine_ = 0;
+    if (cluster_ok_) {
+      int K = 4;
+      for (;; K *= 2) {
+        cg_layout(y, mg_nlev_, K, K, (int)sizeof(T), CG_CLUSTER, kCgSmem);
+        if (K == kCgCluster || (y.bytes <= kCgSmem && M <= K * kCgPerCluster * share)) break;
+      }
+      if (y.bytes <= kCgSmem) {
+        cg_engine_ = CG_CLUSTER + 1;
+        cg_blocks_ = K;
+      } else if (M <= kCgHybridMax) {
+        const int want = (M + kCgPerBlock * share - 1) / (kCgPerBlock * share);
+        K = std::max(2 * kCgCluster, std::min(hyb_blocks_, (want + kCgCluster - 1) / kCgCluster * kCgCluster));
+        K = std::min(K, hyb_blocks_);
+        cg_layout(y, mg_nlev_, K, kCgCluster, (int)sizeof(T), CG_HYBRID, kCgSmem);
+        if (y.bytes <= kCgSmem) {
+          cg_engine_ = CG_HYBRID + 1;
+          cg_blocks_ = K;
+        }
+      }
     }
-    if (cluster_ok_ && y.bytes <= kCgSmem) {
-      cg_engine_ = 1;
-      cg_blocks_ = K;
-    } else {
-      cg_engine_ = 2;
+    if (cg_engine_ == 0) {
+      cg_engine_ = CG_GRID + 1;
       cg_blocks_ = std::max(1, std::min(cg_sms(), (M + kCgPerBlock * share - 1) / (kCgPerBlock * share)));
     }
-    cg_make_layout(cg_engine_ == 1 ? cg_blocks_ : kCgCluster, cg_engine_ == 2 ? cg_blocks_ : cg_sms());
+    cg_make_layout();
   }
 
   // Level l coarsens the grid 2x per axis l times (z only in 3D) while every coarsened
@@ -1599,14 +1630,19 @@ template <typename T> class Stepper : public PlanBase {
   int nsm_ = 1;
   int tune_zb_ = 0, tune_kb_ = 0;           // requested pass-A z-planes / pass-B pencil blocks (0: default)
   int tune_direct_ = 0;                      // 1: direct pass-A loads/stores (no tensor-copy staging)
-  // band solve: blocks, nodes per block of the grid engine, and the grid size up to which a band
-  // of unknown size may fit the cluster engine
-  static constexpr int kCgCluster = 16, kCgPerBlock = sizeof(T) == 4 ? 1024 : 512, kCgPerCluster = sizeof(T) == 4 ? 256 : 64;
-  static constexpr long long kCgClusterGrid = 1LL << 19;
-  int cg_engine_ = 0, cg_blocks_ = 0;        // frozen band: engine (1 cluster, 2 grid) and blocks; 0: unknown
+  // Band solve: nodes per block; the grid sizes up to which a band of unknown size is tried on the
+  // cluster and on the hybrid engine (a shell is some 6% of the grid), and the frozen band up to
+  // which the hybrid engine's 112 blocks (7 clusters of 16) hold a node per thread.  Solve times,
+  // grid against hybrid engine: 38 k nodes FP32 522 against 360 us, 101 k FP64 742 against 688,
+  // 125 k FP32 288 against 310, 125 k FP64 796 against 945 (fewer blocks than the grid's 152).
+  static constexpr int kCgPerBlock = sizeof(T) == 4 ? 1024 : 512, kCgPerCluster = sizeof(T) == 4 ? 256 : 64;
+  static constexpr long long kCgClusterGrid = 1LL << 19, kCgHybridGrid = 1LL << 20;
+  static constexpr int kCgHybridMax = 112 * 1024;
+  int cg_engine_ = 0, cg_blocks_ = 0;        // frozen band: engine (1 + CG_*) and blocks; 0: unknown
   bool cluster_ok_ = true;
   bool shared_gpu_ = false;                  // other plans run beside this one (a batch): fewer, fuller blocks
-  CGLayout* cg_lay_ = nullptr;               // [0] cluster, [1] grid (device)
+  CGLayout* cg_lay_ = nullptr;               // [0] cluster, [1] grid, [2] hybrid (device)
+  int hyb_blocks_ = 0;                       // blocks of the hybrid engine: all the clusters that fit the GPU
   long long wait_budget_ = 4000000000LL;   // grid barrier: clock cycles before ETD_ETIMEOUT
   long long wait_tries_ = 1LL << 22;       // pass-A tensor copy: mbarrier polls before ETD_ETIMEOUT
   size_t smemA_ = 0, smemB1_ = 0;

@@ -57,3 +57,46 @@ def test_band_solve_sizes_match_oracle(n, kind, prec):
     got = w.cpu().numpy().astype(np.float64)
     assert np.linalg.norm(got - want) / np.linalg.norm(want) < (1e-10 if prec == 0 else 2e-5)
     assert not got[~band].any()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,kind", [((128, 128, 64), "thin"), ((128, 128, 128), "shell"), ((256, 64, 64), "thin")])
+def test_large_band_solve_residual(n, kind, prec):
+    """Bands past one cluster, of a size the host does not know (the hybrid or the grid engine):
+    the solution's own residual, formed by the oracle's operator, and its mean.  FP32: rounding w
+    to FP32 alone leaves a residual of eps32 max(diag) |w| / |b|, below 1e-3 here."""
+    p = _params(n, prec)
+    rng = np.random.default_rng(2)
+    dt = np.float64 if prec == 0 else np.float32
+    phi = _membrane(p, kind, rng).astype(dt).astype(np.float64)
+    band, g = obm.band_mask(phi, p.band_mask_hi), omodel.g_loc(phi)
+    f = np.where(band, rng.uniform(-1.0, 1.0, size=p.shape), 0.0).astype(dt).astype(np.float64)
+    plan = Plan(p.replace(cg_rtol=1e-12 if prec == 0 else 1e-6))
+    dev = lambda a: torch.tensor(a, dtype=plan.dtype, device=DEV)  # noqa: E731
+    w = torch.zeros(p.shape, dtype=plan.dtype, device=DEV)
+    it, res = plan.nonlocal_solve(dev(phi), dev(f), w)
+    got = w.cpu().numpy().astype(np.float64)
+    b = np.where(band, f - f[band].mean(), 0.0)
+    r = b - obm.apply_neg_lap(got, obm.face_coeffs(g, band), p.h)
+    assert it > 0 and res <= (1e-12 if prec == 0 else 1e-6)
+    assert np.linalg.norm(r) <= (1e-10 if prec == 0 else 1e-3) * np.linalg.norm(b)
+    assert abs(got[band].mean()) <= (1e-12 if prec == 0 else 1e-5) * np.abs(got).max() and not got[~band].any()
+
+
+@pytest.mark.parametrize("n,kind,prec,tol", [((64, 64, 64), "shell", 0, 1e-11), ((96, 64, 32), "shell", 0, 1e-11),
+                                             ((64, 64, 64), "shell", 1, 3e-5), ((64, 64, 32), "thin", 1, 3e-5)])
+def test_frozen_band_step_matches_oracle(n, kind, prec, tol):
+    """A frozen band's engine is chosen from its level counts (64^3 shell: the hybrid engine).  The
+    bounds are those of the fixed-membrane step tests."""
+    from oracle import etd as oetd
+    p = _params(n, prec).replace(scheme=1, tau=1e-3, M=100.0)
+    rng = np.random.default_rng(4)
+    dt = np.float64 if prec == 0 else np.float32
+    phi = _membrane(p, kind, rng).astype(dt).astype(np.float64)
+    u = rng.uniform(0.3, 0.7, size=p.shape).astype(dt).astype(np.float64)
+    want = oetd.FixedStepper(p.replace(cg_rtol=1e-13), phi).run(u.copy(), 1)
+    plan = Plan(p)
+    dev = lambda a: torch.tensor(a, dtype=plan.dtype, device=DEV)  # noqa: E731
+    ud = dev(u)
+    plan.step(dev(phi), ud, 1, diag=True)
+    assert np.linalg.norm(ud.cpu().numpy() - want) < tol * np.linalg.norm(want)

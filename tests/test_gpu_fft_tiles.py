@@ -34,19 +34,21 @@ def test_transforms_match_numpy(n, prec, tol):
     assert float((back.double() - f.double()).norm()) < tol * float(f.double().norm())
 
 
-@pytest.mark.parametrize("prec", [0, 1])
-def test_r1_of_an_unaligned_field_is_the_same(prec):
-    """u one element past a 16-byte boundary takes the one-point loads: the same bits."""
+@pytest.mark.parametrize("prec,tol", [(0, 1e-11), (1, 2e-5)])
+def test_r1_of_an_unaligned_field_matches_oracle(prec, tol):
+    """u one element past a 16-byte boundary takes the one-point loads (the bounds of the aligned
+    R1 test; not bit for bit, the volume in R1 being a sum of atomics)."""
+    from oracle import model as omodel
     p, phi, u, _ = wl.workload("c3", n=32, precision=prec)
-    plan = Plan(p.replace(A0=1.0))
+    p = p.replace(A0=omodel.volume(phi, p) - 0.05)
+    plan = Plan(p)
     dt = plan.dtype
     phid = torch.tensor(phi, dtype=dt, device=DEV)
-    ud = torch.tensor(u, dtype=dt, device=DEV)
     buf = torch.zeros(u.size + 1, dtype=dt, device=DEV)
-    buf[1:] = ud.reshape(-1)
+    buf[1:] = torch.tensor(u, dtype=dt, device=DEV).reshape(-1)
     uu = buf[1:].view(u.shape)
     assert uu.data_ptr() % 16 != 0
-    a, b = torch.zeros_like(phid), torch.zeros_like(phid)
-    plan.remainder(1, phid, None, ud, a)
-    plan.remainder(1, phid, None, uu, b)
-    assert torch.equal(a, b)
+    out = torch.zeros_like(phid)
+    plan.remainder(1, phid, None, uu, out)
+    want = omodel.R1(phi, u, p, p.A0)
+    assert np.linalg.norm(out.cpu().numpy() - want) < tol * np.linalg.norm(want)
