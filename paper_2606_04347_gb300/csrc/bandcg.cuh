@@ -122,7 +122,7 @@ struct MGP {
   MGL L[kMGMax];
 };
 
-// Shared-memory layout of a block, from the level counts alone (k_cg_layout, once per band).
+// Shared-memory layout of a block, from the level counts alone (once per band).
 // Distributed levels l < lc: block k owns nodes [k n[l], (k + 1) n[l]); local levels l >= lc are
 // held whole by every block.
 struct CGLayout {
@@ -220,17 +220,19 @@ struct CGCtl2 {
   int KC;                // blocks of a cluster
 };
 
-// One warp per layout: [0] the cluster engine's for clK blocks, [1] the grid engine's for gridK,
-// [2] the hybrid engine's for hybK in clusters of kCgCluster.
+// Layouts of a band: [0] the cluster engine's, [1] the grid engine's, [2] the hybrid engine's in
+// clusters of kCgCluster.
 constexpr int kCgCluster = 16;
 struct CGCounts {
   const int* cnt[kMGMax];
 };
-static __global__ void k_cg_layout(CGCounts cs, int nlev, int tsize, int clK, int gridK, int hybK, int gsmem,
-                                   CGLayout* out) {
+// One warp per layout (the first three warps of the block).
+__device__ inline void cg_layouts(const int* const* cnt, int nlev, int tsize, int clK, int gridK, int hybK, int gsmem,
+                                  CGLayout* out) {
   __shared__ CGLayout y[3];
   const int e = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l < kMGMax) y[e].cnt[l] = l < nlev ? *cs.cnt[l] : 0;
+  if (e >= 3) return;
+  if (l < kMGMax) y[e].cnt[l] = l < nlev ? *cnt[l] : 0;
   __syncwarp();
   if (l == 0) {
     if (e == 0) cg_layout(y[e], nlev, clK, clK, tsize, CG_CLUSTER, kCgSmem);
@@ -240,6 +242,10 @@ static __global__ void k_cg_layout(CGCounts cs, int nlev, int tsize, int clK, in
   __syncwarp();
   for (int k = l; k < (int)(sizeof(CGLayout) / 4); k += 32)
     reinterpret_cast<int*>(out + e)[k] = reinterpret_cast<const int*>(&y[e])[k];
+}
+static __global__ void k_cg_layout(CGCounts cs, int nlev, int tsize, int clK, int gridK, int hybK, int gsmem,
+                                   CGLayout* out) {
+  cg_layouts(cs.cnt, nlev, tsize, clK, gridK, hybK, gsmem, out);
 }
 
 // ---- shared-memory access by 32-bit address -------------------------------------------------

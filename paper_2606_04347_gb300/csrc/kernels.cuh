@@ -915,8 +915,10 @@ template <typename T> struct CGVec {
 template <typename T>
 __global__ void k_cg_setup(Geo g, ModelC<T> mc, const int* __restrict__ idx, const int* __restrict__ count,
                            const unsigned char* __restrict__ mask, const int* __restrict__ bmap,
-                           const T* __restrict__ G, CGVec<T> v) {
+                           const T* __restrict__ G, CGVec<T> v, int* cc_flags) {
   const int M = *count;
+  // labelling: component count, fallback flag, barrier counters of the fallback
+  if (blockIdx.x == 0 && threadIdx.x < 4) cc_flags[threadIdx.x] = 0;
   const int nd = g.nz > 1 ? 6 : 4;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
     const int p = idx[i];
@@ -979,59 +981,6 @@ __device__ __forceinline__ int cc_root(int* __restrict__ parent, int v) {
   return cur;
 }
 
-// Each node starts as a child of its smallest band neighbour (or of itself), which leaves a
-// forest with one tree per local minimum of the index over the band; linking then only has to
-// merge those trees.
-template <typename T>
-__global__ void k_cc_init(const int* __restrict__ count, CGVec<T> v, int* __restrict__ parent, const int* fallback) {
-  if (!*fallback) return;
-  const int M = *count;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-    int m = i;
-#pragma unroll
-    for (int f = 0; f < 6; ++f) m = min(m, v.nb[f * v.cap + i]);
-    parent[i] = m;
-  }
-}
-
-template <typename T>
-__global__ void k_cc_link(const int* __restrict__ count, CGVec<T> v, int* __restrict__ parent, int* status,
-                          const int* fallback) {
-  if (!*fallback) return;
-  const int M = *count;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int f = 0; f < 6; f += 2) {       // the + faces: every band edge is seen from one end
-      const int j = v.nb[f * v.cap + i];
-      if (j == i) continue;
-      int a = cc_root(parent, i), b = cc_root(parent, j);
-      for (int tries = 0; a != b; ++tries) {
-        if (tries > M) {                   // cannot happen; guards the loop bound
-          atomicCAS(status, 0, 8);
-          return;
-        }
-        const int hi = a > b ? a : b, lo = a > b ? b : a;
-        const int old = atomicCAS(parent + hi, hi, lo);
-        if (old == hi) break;
-        a = cc_root(parent, old);
-        b = lo;
-      }
-    }
-  }
-}
-
-// Full compression and a compact id per root (arbitrary order).
-static __global__ void k_cc_roots(const int* __restrict__ count, int* __restrict__ parent, int* __restrict__ cid,
-                                  int* __restrict__ ncomp, const int* fallback) {
-  if (!*fallback) return;
-  const int M = *count;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-    const int r = cc_root(parent, i);
-    parent[i] = r;
-    if (r == i) cid[i] = atomicAdd(ncomp, 1);
-  }
-}
-
 // Per-component sums of one pass over the band: components below kCompShared accumulate in
 // shared memory (one global atomic per block and component), others per warp group (lanes
 // holding the same component combine their values, one atomic per group).  Every thread of
@@ -1064,161 +1013,6 @@ struct CompAcc {
     __syncthreads();
   }
 };
-
-// Node components and component sizes.  A band of one component needs neither: the solve
-// then removes the plain mean, and only the size is written.
-static __global__ void k_cc_label(const int* __restrict__ count, const int* __restrict__ parent,
-                                  const int* __restrict__ cid, const int* __restrict__ ncomp, int* __restrict__ comp,
-                                  double* __restrict__ csize, int* status, const int* fallback) {
-  __shared__ double sh[kCompShared];
-  if (!*fallback) return;
-  const int M = *count;
-  const int C = *ncomp;
-  if (C > kCompCap) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(status, 0, 8);
-    return;
-  }
-  if (C <= 1) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) csize[0] = (double)M;
-    return;
-  }
-  CompAcc acc{sh, csize, C};
-  acc.begin();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-    const int c = cid[parent[i]];
-    comp[i] = c;
-    acc.add(c, 1.0);
-  }
-  acc.end();
-}
-
-// Components from the multigrid hierarchy of the band solve.  A node of level l+1 is a 2x2x2
-// cell of level-l nodes, and two level-(l+1) nodes are coupled exactly when a level-l coupling
-// crosses between them.  If the children of every cell are connected inside the cell, the
-// components of each level are the components of the next coarser one, so labelling the
-// coarsest level (at most kCCCoarse nodes, one block) and following each band node's chain of
-// parents gives the band's components.  A cell whose children split inside it, or a coarsest
-// level that does not fit one block, sets the fallback flag and the union-find above runs.
-constexpr int kCCCoarse = 1024;
-constexpr int kCCMaxLev = 7;
-
-struct CCLevel {
-  const int* cnt;     // node count
-  const int* nb;      // neighbour node of each face (the node itself where there is no coupling)
-  const int* child;   // child[k * cap + I]: node of the finer level in sub-cell k, -1 if none
-  const int* agg;     // parent node on the next coarser level
-  int cap;
-};
-struct CCLevels {
-  int nlev, is3d;
-  CCLevel L[kCCMaxLev];
-};
-
-// Are the children of each cell connected inside it?  Sub-cell k = a + 2 b + 4 c (x, y, z bits);
-// its in-cell neighbour across axis d is k ^ (1 << d), reached through face 2 d (+) when bit d of
-// k is 0 and face 2 d + 1 (-) when it is 1.
-static __global__ void k_cc_check(CCLevels lv, int* fallback) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-  const int nax = lv.is3d ? 3 : 2;
-  for (int l = 0; l + 1 < lv.nlev; ++l) {
-    const CCLevel& F = lv.L[l];
-    const CCLevel& Cl = lv.L[l + 1];
-    const int Mc = *Cl.cnt;
-    for (int I = tid; I < Mc; I += nth) {
-      int ch[8];
-      unsigned pres = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        ch[k] = Cl.child[k * Cl.cap + I];
-        if (ch[k] >= 0) pres |= 1u << k;
-      }
-      if (__popc(pres) <= 1) continue;
-      unsigned adj[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        adj[k] = 0;
-        if (!((pres >> k) & 1)) continue;
-        for (int d = 0; d < nax; ++d) {
-          const int k2 = k ^ (1 << d);
-          if (!((pres >> k2) & 1)) continue;
-          const int f = 2 * d + ((k >> d) & 1);
-          if (F.nb[f * F.cap + ch[k]] == ch[k2]) adj[k] |= 1u << k2;
-        }
-      }
-      unsigned r = pres & (~pres + 1u);   // lowest present sub-cell
-#pragma unroll
-      for (int it = 0; it < 3; ++it) {    // the cube graph has diameter 3
-        unsigned nr = r;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if ((r >> k) & 1) nr |= adj[k];
-        r = nr;
-      }
-      if (r != pres) atomicExch(fallback, 1);
-    }
-  }
-}
-
-// Label the coarsest level in one block: min-label propagation with pointer jumping (bounded
-// by the node count), compact ids of the roots, the component count.
-static __global__ void __launch_bounds__(kCCCoarse) k_cc_coarsest(CCLevels lv, int* __restrict__ ccL,
-                                                                  int* __restrict__ ncomp, int* fallback) {
-  __shared__ int lab[kCCCoarse];
-  __shared__ int cid[kCCCoarse];
-  __shared__ int nroot;
-  if (*(volatile int*)fallback) return;
-  const CCLevel& L = lv.L[lv.nlev - 1];
-  const int M = *L.cnt;
-  if (M > kCCCoarse) {
-    if (threadIdx.x == 0) atomicExch(fallback, 1);
-    return;
-  }
-  const int i = threadIdx.x;
-  if (i < M) lab[i] = i;
-  if (i == 0) nroot = 0;
-  __syncthreads();
-  for (int it = 0; it <= M; ++it) {
-    int m = i < M ? lab[i] : 0;
-    if (i < M) {
-      for (int f = 0; f < 6; ++f) {
-        const int j = L.nb[f * L.cap + i];
-        if (j != i) m = min(m, lab[j]);
-      }
-      m = min(m, lab[m]);
-    }
-    __syncthreads();
-    const bool ch = i < M && m < lab[i];
-    if (ch) lab[i] = m;
-    if (!__syncthreads_or(ch)) break;
-  }
-  if (i < M && lab[i] == i) cid[i] = atomicAdd(&nroot, 1);
-  __syncthreads();
-  if (i < M) ccL[i] = cid[lab[i]];
-  if (i == 0) *ncomp = nroot;
-}
-
-// Each band node's component through its chain of parents; the component sizes.
-static __global__ void k_cc_down(CCLevels lv, const int* __restrict__ ccL, const int* __restrict__ ncomp,
-                                 int* __restrict__ comp, double* __restrict__ csize, const int* fallback) {
-  __shared__ double sh[kCompShared];
-  if (*fallback) return;
-  const int M = *lv.L[0].cnt;
-  const int C = *ncomp;
-  if (C <= 1) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) csize[0] = (double)M;
-    return;
-  }
-  CompAcc acc{sh, csize, C};
-  acc.begin();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-    int j = i;
-    for (int l = 0; l + 1 < lv.nlev; ++l) j = lv.L[l].agg[j];
-    const int c = ccL[j];
-    comp[i] = c;
-    acc.add(c, 1.0);
-  }
-  acc.end();
-}
 
 struct CGCtl {
   unsigned* bar;        // [0] monotonic arrival count
@@ -1300,163 +1094,5 @@ __device__ __forceinline__ bool grid_sync(const CGCtl& c) {
 // degree-2 Chebyshev polynomial in D^-1 A (the two sweeps commute, so the cycle stays
 // symmetric), and the coarsest level takes an even number of sweeps with the same pair.
 constexpr int kMGMax = 7;
-
-// Multigrid set-up steps, written for any grid-stride partition (t0, ns) so that the large
-// levels run them as grid-wide kernels and the small ones all inside one block.
-
-// Extents of one level's grid (any even sizes; level l halves level l-1 along every axis,
-// z only in 3D).
-struct Ext {
-  int x, y, z;
-};
-// The cell of level l holding flat index p of level l-1.
-__device__ __forceinline__ int mg_cell(int p, Ext f, int is3d, Ext c) {
-  const int X = p % f.x, t = p / f.x, Y = t % f.y, Z = t / f.y;
-  return ((is3d ? Z >> 1 : 0) * c.y + (Y >> 1)) * c.x + (X >> 1);
-}
-
-// mark the cells of level l (extents c) holding nodes of level l-1 (extents f)
-__device__ __forceinline__ void mg_mark_body(const int* __restrict__ list, int M, Ext f, int is3d, Ext c,
-                                             unsigned char* __restrict__ mark, int t0, int ns) {
-#pragma unroll 4
-  for (int i = t0; i < M; i += ns) mark[mg_cell(list[i], f, is3d, c)] = 1;
-}
-
-__device__ __forceinline__ void mg_parent_body(const int* __restrict__ list, int M, Ext f, int is3d, Ext c,
-                                               const int* __restrict__ cmap, int* __restrict__ agg, int t0, int ns) {
-#pragma unroll 4
-  for (int i = t0; i < M; i += ns) agg[i] = cmap[mg_cell(list[i], f, is3d, c)];
-}
-
-// Galerkin couplings of level l from level l-1.
-__device__ __forceinline__ void mg_coarse_body(const int* __restrict__ clist, int M, Ext ec, int is3d,
-                                               const unsigned char* __restrict__ fmark,
-                                               const int* __restrict__ fmap, Ext ef,
-                                               const float* __restrict__ fc, int fcap, const int* __restrict__ cmap,
-                                               float* __restrict__ c, int* __restrict__ nb, float* __restrict__ idg,
-                                               int* __restrict__ child, int cap, int t0, int ns) {
-  for (int I = t0; I < M; I += ns) {
-    const int C = clist[I];
-    const int X = C % ec.x, tq = C / ec.x, Y = tq % ec.y, Z = tq / ec.y;
-    float s[6] = {0, 0, 0, 0, 0, 0};
-    // the 8 children's marks, then their indices, then their couplings: three rounds of
-    // independent loads instead of a dependent chain per child
-    int Fk[8], jk[8];
-    unsigned char mk[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int a = k & 1, b = (k >> 1) & 1, cz = k >> 2;
-      Fk[k] = ((2 * Z + cz) * ef.y + (2 * Y + b)) * ef.x + (2 * X + a);
-      mk[k] = (is3d || cz == 0) ? fmark[Fk[k]] : (unsigned char)0;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) jk[k] = mk[k] ? fmap[Fk[k]] : -1;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int a = k & 1, b = (k >> 1) & 1, cz = k >> 2;
-      const int j = jk[k];
-      child[k * cap + I] = j;
-      if (j < 0) continue;
-      s[a ? 0 : 1] += fc[(a ? 0 : 1) * fcap + j];
-      s[b ? 2 : 3] += fc[(b ? 2 : 3) * fcap + j];
-      if (is3d) s[cz ? 4 : 5] += fc[(cz ? 4 : 5) * fcap + j];
-    }
-    const int xp = X + 1 == ec.x ? 0 : X + 1, xm = X == 0 ? ec.x - 1 : X - 1;
-    const int yp = Y + 1 == ec.y ? 0 : Y + 1, ym = Y == 0 ? ec.y - 1 : Y - 1;
-    const int zp = Z + 1 == ec.z ? 0 : Z + 1, zm = Z == 0 ? ec.z - 1 : Z - 1;
-    const int ncell[6] = {(Z * ec.y + Y) * ec.x + xp, (Z * ec.y + Y) * ec.x + xm, (Z * ec.y + yp) * ec.x + X,
-                          (Z * ec.y + ym) * ec.x + X, (zp * ec.y + Y) * ec.x + X, (zm * ec.y + Y) * ec.x + X};
-    float d = 0;
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      c[f * cap + I] = s[f];
-      nb[f * cap + I] = s[f] > 0.0f ? cmap[ncell[f]] : I;
-      d += s[f];
-    }
-    idg[I] = d > 0.0f ? 1.0f / d : 1.0f;
-  }
-}
-
-static __global__ void k_mg_mark(const int* __restrict__ list, const int* __restrict__ cnt, Ext f, int is3d, Ext c,
-                                 unsigned char* __restrict__ mark) {
-  mg_mark_body(list, *cnt, f, is3d, c, mark, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
-static __global__ void k_mg_parent(const int* __restrict__ list, const int* __restrict__ cnt, Ext f, int is3d, Ext c,
-                                   const int* __restrict__ cmap, int* __restrict__ agg) {
-  mg_parent_body(list, *cnt, f, is3d, c, cmap, agg, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
-static __global__ void k_mg_coarse(const int* __restrict__ clist, const int* __restrict__ ccnt, Ext ec, int is3d,
-                            const unsigned char* __restrict__ fmark, const int* __restrict__ fmap, Ext ef,
-                            const float* __restrict__ fc, int fcap, const int* __restrict__ cmap, float* __restrict__ c,
-                            int* __restrict__ nb, float* __restrict__ idg, int* __restrict__ child, int cap) {
-  mg_coarse_body(clist, *ccnt, ec, is3d, fmark, fmap, ef, fc, fcap, cmap, c, nb, idg, child, cap,
-                    blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-}
-
-// One level's arrays for the single-block set-up of the small levels.
-struct MGSetLevel {
-  Ext e;
-  int cap;
-  int* cnt;
-  int* list;
-  int* map;
-  unsigned char* mark;
-  float* c;
-  int* nb;
-  float* idg;
-  int* agg;
-  int* child;
-};
-
-struct MGSetTail {
-  int first, nlev, is3d;
-  MGSetLevel L[kMGMax];
-};
-
-// Levels first..nlev-1 built in order by one block of 1024 threads: mark, compact (one
-// contiguous chunk of cells per thread, block-wide exclusive scan), parent map of the
-// finer level, Galerkin couplings.  The finer level of `first` is complete on entry.
-static __global__ void __launch_bounds__(1024) k_mg_setup_tail(MGSetTail a) {
-  __shared__ int part[1024];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int l = a.first; l < a.nlev; ++l) {
-    const MGSetLevel& F = a.L[l - 1];
-    const MGSetLevel& L = a.L[l];
-    for (int i = tid; i < L.cap; i += nt) L.mark[i] = 0;
-    __syncthreads();
-    const int MF = *F.cnt;
-    mg_mark_body(F.list, MF, F.e, a.is3d, L.e, L.mark, tid, nt);
-    __syncthreads();
-    const int per = (L.cap + nt - 1) / nt;
-    const int lo = min(L.cap, tid * per), hi = min(L.cap, lo + per);
-    int own = 0;
-#pragma unroll 4
-    for (int i = lo; i < hi; ++i) own += L.mark[i];
-    part[tid] = own;
-    __syncthreads();
-    for (int off = 1; off < nt; off <<= 1) {
-      const int v = tid >= off ? part[tid - off] : 0;
-      __syncthreads();
-      part[tid] += v;
-      __syncthreads();
-    }
-    int pos = part[tid] - own;
-    for (int i = lo; i < hi; ++i)
-      if (L.mark[i]) {
-        L.list[pos] = i;
-        L.map[i] = pos;
-        ++pos;
-      }
-    if (tid == nt - 1) *L.cnt = part[tid];
-    __syncthreads();
-    const int M = part[nt - 1];
-    mg_parent_body(F.list, MF, F.e, a.is3d, L.e, L.map, F.agg, tid, nt);
-    mg_coarse_body(L.list, M, L.e, a.is3d, F.mark, F.map, F.e, F.c, F.cap, L.map, L.c, L.nb,
-                      L.idg, L.child, L.cap, tid, nt);
-    __syncthreads();
-  }
-}
 
 }  // namespace etd

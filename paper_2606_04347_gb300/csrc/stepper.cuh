@@ -9,12 +9,11 @@
 #include "bandcg.cuh"
 #include "kernels.cuh"
 #include "krylov.cuh"
+#include "mgsetup.cuh"
 #include "ops.cuh"
 #include "plan.h"
 
 namespace etd {
-
-static_assert(kCCMaxLev >= kMGMax, "component labelling covers every multigrid level");
 
 // phi_0, phi_1, phi_2 of Sec. 2.2 in FP64: Taylor series below z = 1 (the closed forms
 // cancel there), closed forms through expm1 above.
@@ -354,8 +353,8 @@ template <typename T> class Stepper : public PlanBase {
     cc_parent_ = alloc<int>(g_.n);
     cc_cid_ = alloc<int>(g_.n);
     cc_comp_ = alloc<int>(g_.n);
-    ncomp_ = alloc<int>(2);   // component count, fallback flag of the labelling
-    ETD_CUDA(cudaMemset(ncomp_, 0, 2 * sizeof(int)));
+    ncomp_ = alloc<int>(4);   // component count, fallback flag of the labelling, its barrier counters
+    ETD_CUDA(cudaMemset(ncomp_, 0, 4 * sizeof(int)));
     ccL_ = alloc<int>(kCCCoarse);
     csize_ = alloc<double>(kCompCap);
     csum_ = alloc<double>(2 * kCompCap);
@@ -751,41 +750,42 @@ template <typename T> class Stepper : public PlanBase {
 
   void cg_setup(const T* G) {
     CGVec<T> v = cg_;
-    timed(ETD_K_BAND, 0.0, [&] { k_cg_setup<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, mask_, bmap_, G, v); });
+    timed(ETD_K_BAND, 0.0,
+          [&] { k_cg_setup<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, mask_, bmap_, G, v, ncomp_); });
     mg_setup();
-    cg_make_layout();
     label_components();
     ETD_CUDA(cudaGetLastError());
   }
 
-  // Connected components of the band (their count, each node's component, their sizes): from
-  // the multigrid hierarchy when every aggregate is connected inside its cell, else by the
+  // Connected components of the band (each node's component, their sizes; the count is known):
+  // from the multigrid hierarchy when every aggregate is connected inside its cell, else by the
   // union-find over the band (both enqueued; the one not needed returns at once).
   void label_components() {
-    CGVec<T> v = cg_;
     CCLevels lv{};
     lv.nlev = mg_nlev_;
-    lv.is3d = g_.nz > 1;
     for (int l = 0; l < mg_nlev_; ++l) {
-      const HostLevel& H = lv_[l];
-      CCLevel& C = lv.L[l];
-      C.cap = H.cap;
-      C.agg = H.agg;
-      C.cnt = l == 0 ? count_ : H.cnt;
-      C.nb = l == 0 ? cg_.nb : H.nb;
-      C.child = l == 0 ? nullptr : H.child;
+      lv.cnt[l] = l == 0 ? count_ : lv_[l].cnt;
+      lv.agg[l] = lv_[l].agg;
     }
+    lv.tsize = (int)sizeof(T);
+    lv.clK = cg_default_blocks(CG_CLUSTER);
+    lv.gridK = cg_default_blocks(CG_GRID);
+    lv.hybK = std::max(cg_default_blocks(CG_HYBRID), kCgCluster);
+    lv.gsmem = grid_smem();
+    lv.lay = cg_lay_;
+    CGCtl c{};
+    c.bar = reinterpret_cast<unsigned*>(ncomp_ + 2);
+    c.status = status_;
+    c.budget = wait_budget_;
+    const int* cnt = count_;
+    const int* nb = cg_.nb;
+    int cap = cg_.cap;
+    int* nc = ncomp_;
+    const int* fb = ncomp_ + 1;
     timed(ETD_K_BAND, 0.0, [&] {
-      ETD_CUDA(cudaMemsetAsync(ncomp_, 0, 2 * sizeof(int), st_));   // count, fallback flag
-      ETD_CUDA(cudaMemsetAsync(csize_, 0, sizeof(double) * kCompCap, st_));
-      int* fb = ncomp_ + 1;
-      if (mg_nlev_ > 1) k_cc_check<<<nsm_ * 2, 256, 0, st_>>>(lv, fb);
-      k_cc_coarsest<<<1, kCCCoarse, 0, st_>>>(lv, ccL_, ncomp_, fb);
-      k_cc_down<<<nsm_ * 4, 256, 0, st_>>>(lv, ccL_, ncomp_, cc_comp_, csize_, fb);
-      k_cc_init<T><<<nsm_ * 4, 256, 0, st_>>>(count_, v, cc_parent_, fb);
-      k_cc_link<T><<<nsm_ * 4, 256, 0, st_>>>(count_, v, cc_parent_, status_, fb);
-      k_cc_roots<<<nsm_ * 4, 256, 0, st_>>>(count_, cc_parent_, cc_cid_, ncomp_, fb);
-      k_cc_label<<<nsm_ * 4, 256, 0, st_>>>(count_, cc_parent_, cc_cid_, ncomp_, cc_comp_, csize_, status_, fb);
+      k_cc_down<<<nsm_ * 4 + 1, 256, 0, st_>>>(lv, ccL_, ncomp_, cc_comp_, csize_, fb);
+      void* args[] = {&cnt, &nb, &cap, &cc_parent_, &cc_cid_, &nc, &cc_comp_, &csize_, &fb, &c};
+      ETD_CUDA(cudaLaunchCooperativeKernel((const void*)k_cc_union, nsm_ * 4, 256, args, 0, st_));
     });
   }
 
@@ -959,7 +959,7 @@ template <typename T> class Stepper : public PlanBase {
       if (y.bytes <= kCgSmem) {
         cg_engine_ = CG_CLUSTER + 1;
         cg_blocks_ = K;
-      } else if (M <= kCgHybridMax) {
+      } else if (M <= kCgHybridMax * (shared_gpu_ ? 2 : 1)) {
         const int want = (M + kCgPerBlock * share - 1) / (kCgPerBlock * share);
         K = std::max(2 * kCgCluster, std::min(hyb_blocks_, (want + kCgCluster - 1) / kCgCluster * kCgCluster));
         K = std::min(K, hyb_blocks_);
@@ -1017,12 +1017,13 @@ template <typename T> class Stepper : public PlanBase {
   }
 
   // Coarse levels for the current band (level 0 = idx_, count_, mask_, bmap_, cg_).  Levels
-  // whose full grid has more than 2^15 cells use grid-wide kernels; the rest are built by
-  // one single-block launch (they are too small to fill the GPU, and launch gaps dominate).
+  // whose full grid has more than 2^15 cells use grid-wide kernels; the rest, the labels of the
+  // coarsest one are one launch of a single cluster (they are too small to
+  // fill the GPU, and launch gaps dominate).
   void mg_setup() {
     const int is3d = g_.nz > 1;
     int l = 1;
-    for (; l < mg_nlev_ && lv_[l].cap > (1 << 15); ++l) {
+    for (; l < mg_nlev_ && lv_[l].cap > kTailCells; ++l) {
       HostLevel& L = lv_[l];
       const HostLevel& F = lv_[l - 1];
       const int* flist = l == 1 ? idx_ : F.list;
@@ -1030,6 +1031,7 @@ template <typename T> class Stepper : public PlanBase {
       const unsigned char* fmark = l == 1 ? mask_ : F.mark;
       const int* fmap = l == 1 ? bmap_ : F.map;
       const float* fc = l == 1 ? cg_.c32 : F.c;
+      const int* fnb = l == 1 ? cg_.nb : F.nb;
       int* fagg = lv_[l - 1].agg;
       timed(ETD_K_BAND, 0.0, [&] {
         ETD_CUDA(cudaMemsetAsync(L.mark, 0, L.cap, st_));
@@ -1045,45 +1047,27 @@ template <typename T> class Stepper : public PlanBase {
           k_band_scatter<<<L.nblk, kCompactBlock, 0, st_>>>(L.cap, L.mark, L.bcount, L.list, L.map);
         }
         k_mg_parent<<<nsm_ * 4, 256, 0, st_>>>(flist, fcnt, F.ext, is3d, L.ext, L.map, fagg);
-        k_mg_coarse<<<nsm_ * 4, 256, 0, st_>>>(L.list, L.cnt, L.ext, is3d, fmark, fmap, F.ext, fc,
-                                                  F.cap, L.map, L.c, L.nb, L.idg, L.child, L.cap);
+        k_mg_coarse<<<nsm_ * 4, 256, 0, st_>>>(L.list, L.cnt, L.ext, is3d, fmark, fmap, F.ext, fc, fnb, F.cap, L.map,
+                                               L.c, L.nb, L.idg, L.child, L.cap, ncomp_ + 1);
       });
       ETD_CUDA(cudaGetLastError());
     }
-    if (l < mg_nlev_) {
-      MGSetTail a{};
-      a.first = l;
-      a.nlev = mg_nlev_;
-      a.is3d = is3d;
-      for (int k = 0; k < mg_nlev_; ++k) {
-        const HostLevel& H = lv_[k];
-        MGSetLevel& S = a.L[k];
-        S.e = H.ext;
-        S.cap = H.cap;
-        S.agg = H.agg;
-        if (k == 0) {
-          S.cnt = count_;
-          S.list = idx_;
-          S.map = bmap_;
-          S.mark = mask_;
-          S.c = cg_.c32;
-          S.nb = cg_.nb;
-          S.idg = cg_.idg;
-          S.child = nullptr;
-        } else {
-          S.cnt = H.cnt;
-          S.list = H.list;
-          S.map = H.map;
-          S.mark = H.mark;
-          S.c = H.c;
-          S.nb = H.nb;
-          S.idg = H.idg;
-          S.child = H.child;
-        }
-      }
-      timed(ETD_K_BAND, 0.0, [&] { k_mg_setup_tail<<<1, 1024, 0, st_>>>(a); });
-      ETD_CUDA(cudaGetLastError());
+    MGTail a{};
+    a.first = l;
+    a.nlev = mg_nlev_;
+    a.is3d = is3d;
+    for (int k = 0; k < mg_nlev_; ++k) {
+      const HostLevel& H = lv_[k];
+      a.L[k] = k == 0 ? MGSetLevel{H.ext, H.cap, count_, idx_, bmap_, mask_, cg_.c32, cg_.nb, cg_.idg, H.agg, nullptr}
+                      : MGSetLevel{H.ext, H.cap, H.cnt, H.list, H.map, H.mark, H.c, H.nb, H.idg, H.agg, H.child};
     }
+    a.ccL = ccL_;
+    a.ncomp = ncomp_;
+    a.fallback = ncomp_ + 1;
+    a.csize = csize_;
+    set_smem((const void*)k_mg_tail, kTailSmem);
+    timed(ETD_K_BAND, 0.0, [&] { k_mg_tail<<<kTailBlocks, 1024, kTailSmem, st_>>>(a); });
+    ETD_CUDA(cudaGetLastError());
   }
 
   MGP mgp() const {
@@ -1634,7 +1618,8 @@ template <typename T> class Stepper : public PlanBase {
   // cluster and on the hybrid engine (a shell is some 6% of the grid), and the frozen band up to
   // which the hybrid engine's 112 blocks (7 clusters of 16) hold a node per thread.  Solve times,
   // grid against hybrid engine: 38 k nodes FP32 522 against 360 us, 101 k FP64 742 against 688,
-  // 125 k FP32 288 against 310, 125 k FP64 796 against 945 (fewer blocks than the grid's 152).
+  // 125 k FP32 288 against 310, 125 k FP64 796 against 945 (fewer blocks than the grid's 152).  In a
+  // batch, whose solves run on fewer blocks anyway, up to twice that (8 runs: 18.7 against 17.4 ms).
   static constexpr int kCgPerBlock = sizeof(T) == 4 ? 1024 : 512, kCgPerCluster = sizeof(T) == 4 ? 256 : 64;
   static constexpr long long kCgClusterGrid = 1LL << 19, kCgHybridGrid = 1LL << 20;
   static constexpr int kCgHybridMax = 112 * 1024;
