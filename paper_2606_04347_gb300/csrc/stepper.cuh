@@ -481,6 +481,8 @@ template <typename T> class Stepper : public PlanBase {
     if (kry_mem_) cudaFree(kry_mem_);
     kry_mem_ = nullptr;
     kry_cap_ = 0;
+    if (khost_) cudaFreeHost(khost_);
+    khost_ = nullptr;
     if (fork_ev_) cudaEventDestroy(fork_ev_);
     if (join_ev_) cudaEventDestroy(join_ev_);
     if (side_) cudaStreamDestroy(side_);
@@ -1331,6 +1333,11 @@ template <typename T> class Stepper : public PlanBase {
   // Krylov workspace for the frozen band of fixed_count_ nodes: the Lanczos basis
   // (kKrylovMax + 1 vectors), w, R0, b, V~, g^{1/2}, g^{-1/2} (compact) and FP64 scalars.
   void krylov_setup() {
+    if (!khost_ && cudaMallocHost(&khost_, sizeof(double) * (2 * kKrylovChunk + 1 + kKrylovMax)) != cudaSuccess) {
+      cudaGetLastError();
+      khost_ = nullptr;
+      throw Error(ETD_ENOMEM, "pinned Krylov buffer does not fit");
+    }
     const long long M = std::max(fixed_count_, 1);
     if (M > kry_cap_) {
       if (kry_mem_) ETD_CUDA(cudaFree(kry_mem_));
@@ -1378,10 +1385,12 @@ template <typename T> class Stepper : public PlanBase {
     c.budget = wait_budget_;
     ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
     auto k = k_lanczos<T>;
-    int per = 0;
-    ETD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 1024, 0));
-    if (per < 1) throw Error(ETD_ECUDA, "Lanczos kernel cannot be resident");
-    const int grid = std::max(1, std::min(nsm_, (fixed_count_ + 2047) / 2048));
+    // Nodes spread over all SMs before they fill blocks: the FP64 work of a node on 2 operations a
+    // clock and SM, and block sums over as few warps as hold nodes (5852 nodes FP64, 8 steps: 3
+    // blocks of 1024 184 us, 46 of 128 58 us; a block's threads a power of two from 128 on).
+    int threads = 128;
+    while (threads < 1024 && (long long)threads * nsm_ < fixed_count_) threads *= 2;
+    const int grid = std::max(1, std::min(nsm_, (fixed_count_ + threads - 1) / threads));
     const int* cnt = count_;
     T* V = kV_;
     int ld = kld_;
@@ -1390,7 +1399,7 @@ template <typename T> class Stepper : public PlanBase {
     void* args[] = {&cnt, &op, &V, &ld, &w, &al, &be, &acc, &j0, &j1, &c};
     const double bytes = (double)fixed_count_ * (j1 - j0) * (15.0 * sizeof(T) + 24.0);
     timed(ETD_K_KRYLOV, bytes, [&] {
-      ETD_CUDA(cudaLaunchCooperativeKernel((const void*)k, grid, 1024, args, 0, st_));
+      ETD_CUDA(cudaLaunchCooperativeKernel((const void*)k, grid, threads, args, 0, st_));
     });
   }
 
@@ -1404,9 +1413,9 @@ template <typename T> class Stepper : public PlanBase {
     ETD_CUDA(cudaMemsetAsync(knrm_, 0, sizeof(double), st_));
     timed(ETD_K_KRYLOV, (double)sizeof(T) * fixed_count_,
           [&] { k_band_norm2<T><<<nb, 256, 0, st_>>>(count_, x, knrm_); });
-    double n2 = 0.0;
-    ETD_CUDA(cudaMemcpyAsync(&n2, knrm_, sizeof(double), cudaMemcpyDeviceToHost, st_));
+    ETD_CUDA(cudaMemcpyAsync(khost_, knrm_, sizeof(double), cudaMemcpyDeviceToHost, st_));
     ETD_CUDA(cudaStreamSynchronize(st_));
+    const double n2 = khost_[0];
     if (!std::isfinite(n2)) throw Error(ETD_ENONFINITE, "non-finite value in a Krylov start vector");
     if (n2 == 0.0) return 0;
     const double beta0 = std::sqrt(n2);
@@ -1420,9 +1429,20 @@ template <typename T> class Stepper : public PlanBase {
     for (;;) {
       const int j1 = std::min(m + kKrylovChunk, kKrylovMax);
       lanczos(m, j1);
-      ETD_CUDA(cudaMemcpyAsync(ha + m, kal_ + m, sizeof(double) * (j1 - m), cudaMemcpyDeviceToHost, st_));
-      ETD_CUDA(cudaMemcpyAsync(hb + m, kbe_ + m, sizeof(double) * (j1 - m), cudaMemcpyDeviceToHost, st_));
-      sync_check();
+      // one wait a chunk: the coefficients and the status word through pinned memory (copies to
+      // pageable memory wait one by one)
+      double* h = khost_;
+      ETD_CUDA(cudaMemcpyAsync(h, kal_ + m, sizeof(double) * (j1 - m), cudaMemcpyDeviceToHost, st_));
+      ETD_CUDA(cudaMemcpyAsync(h + kKrylovChunk, kbe_ + m, sizeof(double) * (j1 - m), cudaMemcpyDeviceToHost, st_));
+      int* hs = reinterpret_cast<int*>(h + 2 * kKrylovChunk);
+      ETD_CUDA(cudaMemcpyAsync(hs, status_, sizeof(int), cudaMemcpyDeviceToHost, st_));
+      ETD_CUDA(cudaGetLastError());
+      ETD_CUDA(cudaStreamSynchronize(st_));
+      check_status(*hs);
+      for (int k = m; k < j1; ++k) {
+        ha[k] = h[k - m];
+        hb[k] = h[kKrylovChunk + k - m];
+      }
       dim = j1;
       bool invariant = false;
       for (int k = m; k < j1; ++k) {
@@ -1443,9 +1463,10 @@ template <typename T> class Stepper : public PlanBase {
         throw Error(ETD_ENOTCONV, "the Krylov space of phi_j(tau L) did not converge within 128 Lanczos steps");
       m = j1;
     }
-    for (double& v : y) v *= P_.tau * beta0;
-    ETD_CUDA(cudaMemcpyAsync(ky_, y.data(), sizeof(double) * dim, cudaMemcpyHostToDevice, st_));
-    ETD_CUDA(cudaStreamSynchronize(st_));   // y is a host temporary
+    // the weights' pinned buffer is free again: every call waits for its stream before this copy
+    double* hy = khost_ + 2 * kKrylovChunk + 1;
+    for (int k = 0; k < dim; ++k) hy[k] = y[k] * P_.tau * beta0;
+    ETD_CUDA(cudaMemcpyAsync(ky_, hy, sizeof(double) * dim, cudaMemcpyHostToDevice, st_));
     kry_dim_max_ = std::max(kry_dim_max_, dim);
     return dim;
   }
@@ -1681,6 +1702,7 @@ template <typename T> class Stepper : public PlanBase {
   // frozen band size and the Krylov workspace of the g^{1/2}-split scheme
   int fixed_count_ = 0;
   void* kry_mem_ = nullptr;
+  double* khost_ = nullptr;   // pinned: coefficients of a chunk, status word, combination weights
   long long kry_cap_ = 0;
   int kld_ = 0, kry_dim_max_ = 0;
   T *kV_ = nullptr, *kw_ = nullptr, *kR0_ = nullptr, *kb_ = nullptr, *kVt_ = nullptr, *ksg_ = nullptr, *kisg_ = nullptr;
