@@ -176,8 +176,8 @@ struct MGTail {
 // in 3D an eighth, of the cells of the finer one), the scan's warp sums, then the labels.
 constexpr int kTailSmem = 2 * 2 * 4 * (kTailCells / 32) + 2 * kTailCells + 2 * kTailCells / 4 + 128;
 
-// Every block of the cluster numbers all the cells (the same bitmap in each: no exchange), and
-// they share the nodes' parents and couplings, some 70 scattered loads and stores a node.
+// Every block of the cluster numbers all the cells (the same bitmap in each); they share the
+// marking, the nodes' parents and their couplings, some 70 scattered loads and stores a node.
 constexpr int kTailBlocks = 8;
 __device__ __forceinline__ void tail_barrier() {   // hardware barrier of the cluster, global writes included
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -213,22 +213,23 @@ static __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(102
     auto rank = [&](int C) { return (int)(P[C >> 5] + __popc(W[C >> 5] & ((1u << (C & 31)) - 1u))); };
     W[tid] = 0;
     __syncthreads();
-    // neighbouring nodes share words: one atomic per word and warp (one per node, all on a few
-    // words, took 30 of the kernel's 40 us)
-    for (int i0 = 0; i0 < MF; i0 += 4096) {
-      int C[4];
+    // each block marks its share of the finer nodes; the bitmaps are then or-ed together
+    for (int i = g0; i < MF; i += gs) {
+      const int C = cell(i);
+      if (!((W[C >> 5] >> (C & 31)) & 1u)) atomicOr(&W[C >> 5], 1u << (C & 31));
+    }
+    tail_barrier();
+    {
+      unsigned w = 0;
+      const uint32_t mine = smem_u32(W + tid);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + 1024 * u + tid;
-        C[u] = i < MF ? cell(i) : -1;
+      for (int k = 0; k < kTailBlocks; ++k) {
+        unsigned x;
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(mapa_u32(mine, k)));
+        w |= x;
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int w = C[u] >= 0 ? C[u] >> 5 : -1;
-        const unsigned grp = __match_any_sync(0xffffffffu, w);
-        const unsigned bits = __reduce_or_sync(grp, w >= 0 ? 1u << (C[u] & 31) : 0u);
-        if (w >= 0 && lane == __ffs(grp) - 1) atomicOr(&W[w], bits);
-      }
+      tail_barrier();   // every block has read before any overwrites its bitmap
+      W[tid] = w;
     }
     __syncthreads();
     {
@@ -259,17 +260,27 @@ static __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(102
     const int M = cnts[l];
 #pragma unroll 4
     for (int i = g0; i < MF; i += gs) F.agg[i] = rank(cell(i));
-    for (int I = g0; I < M; I += gs)
-      mg_coarse_node(
-          I, (int)lst[I], e, a.is3d, fe,
-          [&](int C) -> int {
-            if (top) {
-              const int m = F.map[C];
-              return F.mark[C] ? m : -1;
-            }
-            return (FW[C >> 5] >> (C & 31)) & 1u ? (int)(FP[C >> 5] + __popc(FW[C >> 5] & ((1u << (C & 31)) - 1u))) : -1;
-          },
-          F.c, F.nb, F.cap, rank, L.c, L.nb, L.idg, L.child, L.cap, a.fallback);
+    if (top) {
+      const int* __restrict__ fmap = F.map;
+      const unsigned char* __restrict__ fmark = F.mark;
+      for (int I = g0; I < M; I += gs)
+        mg_coarse_node(
+            I, (int)lst[I], e, a.is3d, fe,
+            [&](int C) {
+              const int m = fmap[C];
+              return fmark[C] ? m : -1;
+            },
+            F.c, F.nb, F.cap, rank, L.c, L.nb, L.idg, L.child, L.cap, a.fallback);
+    } else {
+      for (int I = g0; I < M; I += gs)
+        mg_coarse_node(
+            I, (int)lst[I], e, a.is3d, fe,
+            [&](int C) {
+              const unsigned w = FW[C >> 5];
+              return (w >> (C & 31)) & 1u ? (int)(FP[C >> 5] + __popc(w & ((1u << (C & 31)) - 1u))) : -1;
+            },
+            F.c, F.nb, F.cap, rank, L.c, L.nb, L.idg, L.child, L.cap, a.fallback);
+    }
     tail_barrier();
   }
   if (blockIdx.x != 0) return;
