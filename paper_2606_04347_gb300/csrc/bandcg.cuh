@@ -43,9 +43,6 @@ __device__ __forceinline__ float2 make_uw(float u, float w) { return make_float2
 __device__ __forceinline__ double2 make_uw(double u, double w) { return make_double2(u, w); }
 
 // ---- wide scalars: double-float for FP32 storage, FP64 otherwise ---------------------------
-template <typename T> struct WideOf;
-template <> struct WideOf<float> { using type = dfloat; };
-template <> struct WideOf<double> { using type = double; };
 __device__ __forceinline__ double wide_d(double a) { return a; }
 __device__ __forceinline__ double wide_d(dfloat a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ double wdiv(double a, double b) { return a / b; }

@@ -49,6 +49,39 @@ __device__ __forceinline__ void block_add(double v, double* dst) {
   }
 }
 
+// The same for a double-float partial (FP32 storage): shuffles and additions on the FP32 pipes,
+// one FP64 addition per block.  A block's 16 warps need 1.3 k clocks for the FP64 form (an FP64
+// warp instruction holds its pipe for 64), 0.3 k for this one; it is a tail of every reduction
+// and of every summing pass-A epilogue.
+__device__ __forceinline__ void block_add(dfloat v, double* dst) {
+  __shared__ dfloat ws[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = v + dfloat(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o));
+  __syncthreads();
+  if (lane == 0) ws[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    const int nw = (blockDim.x + 31) >> 5;
+    dfloat t = lane < nw ? ws[lane] : dfloat(0.0f, 0.0f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      t = t + dfloat(__shfl_down_sync(0xffffffffu, t.hi, o), __shfl_down_sync(0xffffffffu, t.lo, o));
+    if (lane == 0) atomicAdd(dst, (double)t.hi + (double)t.lo);
+  }
+}
+
+// Wide scalars: double-float for FP32 storage, FP64 otherwise.
+template <typename T> struct WideOf;
+template <> struct WideOf<float> { using type = dfloat; };
+template <> struct WideOf<double> { using type = double; };
+
+// V consecutive values per thread (16-byte loads; V = 1 where a pointer is not 16-byte aligned).
+template <typename T, int V> struct __align__(V * sizeof(T)) VecN {
+  T v[V];
+};
+
 __device__ __forceinline__ void atomic_max_nonneg(double* dst, double v) {
   atomicMax(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)__double_as_longlong(v));
 }
@@ -215,9 +248,6 @@ template <typename T> struct EpiPhiG {
 // aligned), so that six wide loads a thread are in flight: 256^3 FP32 124 -> 88 us for 537 MB.
 // The FP64 form is bound by the FP64 pipe (70 instructions a point with its two quotients by
 // eps_phi and one by eps_u; 128^3 296 us) and multiplies by reciprocals instead.
-template <typename T, int V> struct __align__(V * sizeof(T)) VecN {
-  T v[V];
-};
 template <typename T> __device__ __forceinline__ T quot(T a, T b, T ib) {
   if constexpr (sizeof(T) == 8) return a * ib;
   else return a / b;
@@ -421,6 +451,10 @@ template <typename T> struct CompSum {
     hi = s;
   }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ typename WideOf<T>::type wide() const {
+    if constexpr (sizeof(T) == 4) return dfloat(hi, lo);
+    else return hi + lo;
+  }
 };
 
 // ubar = hi + lo in the storage precision (lo = 0 in FP64).
@@ -450,47 +484,52 @@ __device__ __forceinline__ void add_mass(CompSum<double>& cs, double x, double g
 
 // mode 0: sum a ; 1: sum G (u - ubar) ; 2: sum G (f(u) - ubar).  FP64 storage sums in FP64;
 // FP32 storage forms each term to about twice FP32 precision (ubar split into hi + lo, the
-// product's rounding error from an FMA) and sums with CompSum.
-template <typename T>
-__global__ void k_reduce(long long n, int mode, const T* __restrict__ a, const T* __restrict__ G, double ubar,
-                         double* dst) {
-  if constexpr (sizeof(T) == 8) {
-    double s = 0.0;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-      if (mode == 0) s += (double)a[p];
-      else if (mode == 1) s += (double)G[p] * ((double)a[p] - ubar);
-      else s += (double)G[p] * ((double)find(a[p]) - ubar);
+// product's rounding error from an FMA) and sums with CompSum.  Four blocks per SM at most: each
+// ends in a block sum.
+template <typename T, int V>
+__global__ void __launch_bounds__(256) k_reduce(long long n, int mode, const T* __restrict__ a,
+                                                const T* __restrict__ G, double ubar, double* dst) {
+  using VT = VecN<T, V>;
+  const long long nv = n / V;
+  const Ubar<T> ub = split_ubar<T>(ubar);
+  CompSum<T> cs;
+  double s = 0.0;
+#pragma unroll 2
+  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < nv; p += (long long)gridDim.x * blockDim.x) {
+    const VT av = reinterpret_cast<const VT*>(a)[p];
+    VT gv{};
+    if (mode != 0) gv = reinterpret_cast<const VT*>(G)[p];
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const T x = av.v[k], g = gv.v[k];
+      if constexpr (sizeof(T) == 8) {
+        if (mode == 0) s += x;
+        else s += g * ((mode == 1 ? x : find(x)) - ubar);
+      } else {
+        if (mode == 0) cs.add(x);
+        else add_mass(cs, mode == 1 ? x : find(x), g, ub);
+      }
     }
-    block_add(s, dst);
-    return;
   }
-  const Ubar<float> ub = split_ubar<float>(ubar);
-  CompSum<float> cs;
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
-    if (mode == 0) {
-      cs.add((float)a[p]);
-      continue;
-    }
-    add_mass(cs, mode == 1 ? (float)a[p] : (float)find(a[p]), (float)G[p], ub);
-  }
-  block_add(cs.value(), dst);
+  if constexpr (sizeof(T) == 8) block_add(s, dst);
+  else block_add(cs.wide(), dst);
 }
 
 // ---- inverse-transform epilogues that also form a field sum ------------------------------
 // The volume <phi, 1> and the mass sum G (u - ubar) of Sec. 3.3 (k_reduce modes 0 and 1)
 // accumulate while pass A stores the field: a compensated sum over each row pair a thread
-// stores (Part), folded into FP64 per-thread sums (Acc), one block sum per CTA added
+// stores (Part), folded into wide per-thread sums (Acc), one block sum per CTA added
 // atomically at the end; the field is not read back.  The caller zeroes the targets.
 template <typename T> struct Sums2 {
-  CompSum<T> s0, s1;
+  CompSum<T> s0;
 };
-struct Acc2 {
-  double s0 = 0.0, s1 = 0.0;
+template <typename T> struct Acc2 {
+  typename WideOf<T>::type s0 = typename WideOf<T>::type(0);
 };
 
 template <typename T> struct EpiStoreVol {
   static constexpr bool kPrefetch = false, kSums = true;
-  using Acc = Acc2;
+  using Acc = Acc2<T>;
   using Part = Sums2<T>;
   __device__ void prefetch(long long) const {}
   T* out;
@@ -499,14 +538,14 @@ template <typename T> struct EpiStoreVol {
     out[i] = v;
     a.s0.add(v);
   }
-  __device__ void fold(Part& p, Acc& a) const { a.s0 += p.s0.value(); }
+  __device__ void fold(Part& p, Acc& a) const { a.s0 = a.s0 + p.s0.wide(); }
   __device__ void finish(Acc& a) const { block_add(a.s0, vol); }
 };
 
 // EpiPhiG plus the volume of phi^{n+1}.
 template <typename T> struct EpiPhiGVol {
   static constexpr bool kPrefetch = false, kSums = true;
-  using Acc = Acc2;
+  using Acc = Acc2<T>;
   using Part = Sums2<T>;
   __device__ void prefetch(long long) const {}
   T* phi;
@@ -519,14 +558,14 @@ template <typename T> struct EpiPhiGVol {
     if (zero) zero[i] = 0;
     a.s0.add(v);
   }
-  __device__ void fold(Part& p, Acc& a) const { a.s0 += p.s0.value(); }
+  __device__ void fold(Part& p, Acc& a) const { a.s0 = a.s0 + p.s0.wide(); }
   __device__ void finish(Acc& a) const { block_add(a.s0, vol); }
 };
 
 // EpiRecover plus the mass sum of (G, u~).
 template <typename T> struct EpiRecoverMass {
   static constexpr bool kPrefetch = true, kSums = true;
-  using Acc = Acc2;
+  using Acc = Acc2<T>;
   using Part = Sums2<T>;
   __device__ void prefetch(long long i) const {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(G + i));
@@ -545,7 +584,7 @@ template <typename T> struct EpiRecoverMass {
     out[i] = o;
     add_mass(a.s0, o, gg, ub);
   }
-  __device__ void fold(Part& p, Acc& a) const { a.s0 += p.s0.value(); }
+  __device__ void fold(Part& p, Acc& a) const { a.s0 = a.s0 + p.s0.wide(); }
   __device__ void finish(Acc& a) const { block_add(a.s0, mass); }
 };
 
@@ -564,7 +603,7 @@ struct ProWiden {
 // edge both keep their relative accuracy in G.  Also clears the R2 field and forms the volume.
 struct EpiPhiIncVol {
   static constexpr bool kPrefetch = true, kSums = true;
-  using Acc = Acc2;
+  using Acc = Acc2<float>;
   using Part = Sums2<float>;
   __device__ void prefetch(long long i) const {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(cur + i));
@@ -586,7 +625,7 @@ struct EpiPhiIncVol {
     if (zero) zero[i] = 0.0f;
     a.s0.add(p.hi);
   }
-  __device__ void fold(Part& p, Acc& a) const { a.s0 += p.s0.value(); }
+  __device__ void fold(Part& p, Acc& a) const { a.s0 = a.s0 + p.s0.wide(); }
   __device__ void finish(Acc& a) const { block_add(a.s0, vol); }
 };
 

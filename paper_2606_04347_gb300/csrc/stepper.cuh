@@ -529,7 +529,11 @@ template <typename T> class Stepper : public PlanBase {
 
   void launch_reduce(int mode, const T* a, const T* G, double* dst) {
     timed(ETD_K_REDUCE, (mode == 0 ? 1 : 2) * fld(), [&] {
-      k_reduce<T><<<grid_for(g_.n), 256, 0, st_>>>(g_.n, mode, a, G, P_.ubar, dst);
+      constexpr int V = 16 / sizeof(T);
+      const bool al = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(G)) & 15) == 0 && g_.n % V == 0;
+      const int nb = (int)std::max<long long>(1, std::min<long long>((g_.n / (al ? V : 1) + 255) / 256, 4LL * nsm_));
+      if (al) k_reduce<T, V><<<nb, 256, 0, st_>>>(g_.n, mode, a, G, P_.ubar, dst);
+      else k_reduce<T, 1><<<nb, 256, 0, st_>>>(g_.n, mode, a, G, P_.ubar, dst);
     });
     ETD_CUDA(cudaGetLastError());
   }
