@@ -130,7 +130,7 @@ struct CGLayout {
   int mat[kMGMax];     // byte offset of the cached matrix (distributed: c, nb code, idg, child code;
                        // local: c, idg, nb, child), -1: read from global memory
   int vec[kMGMax];     // byte offset of b, e, o, t (levels of a cluster, and local levels)
-  int cgv;             // byte offset of x, r, p, q (cluster engine)
+  int cgv;             // byte offset of x, p, q and (FP64) r (cluster engine)
   int c64;             // byte offset of the FP64 couplings, -1: read from global memory
   int agg;             // byte offset of the parents of level lc - 1's own nodes (16-bit), -1: global
   int par;             // hybrid: byte offset of the parent codes of level lg - 1's own nodes
@@ -191,7 +191,7 @@ __host__ __device__ inline void cg_layout(CGLayout& y, int nlev, int K, int KC, 
     const int n = y.n[l];
     if (n > smem / 52) return;   // more than a block holds (and no overflow below)
     y.vec[l] = take(16 * n);
-    if (l == 0) y.cgv = take(4 * tsize * n);
+    if (l == 0) y.cgv = take((tsize == 4 ? 3 : 4) * tsize * n);
     y.mat[l] = take((l > 0 ? 84 : 52) * n);
     if (l == 0 && tsize == 8) y.c64 = take(48 * n);
   }
@@ -315,30 +315,67 @@ template <> struct LevD<false> {  // vectors in global memory, the matrix there 
   const unsigned* pnb;
   const float* pidg;
   const unsigned* pch;
-  const __half* c16;              // streamed level 0 of the FP32 form: couplings of the later sweeps
+  // streamed level 0 of the FP32 form: couplings of the later sweeps; packed form (null: not)
+  const __half* c16;
+  const uint4* pk;                // FP16 couplings and the FP32 inverse diagonal
+  const short4* nd;               // y and z neighbours as offsets (x neighbours are s - 1, s + 1)
   float* g[4];                    // the whole vectors
   int lb;                         // first own node
   __device__ float c(int f, int s, bool half) const {
     return half && c16 ? __half2float(c16[f * cs + s]) : pc[f * cs + s];
   }
   __device__ unsigned nb(int f, int s) const { return pnb[f * cs + s]; }
-  __device__ float idg(int s) const { return pidg[s]; }
+  __device__ float idg(int s) const { return pk ? __uint_as_float(pk[s].w) : pidg[s]; }
   __device__ unsigned child(int k, int s) const { return pch[k * cs + s]; }
   __device__ float own(int v, int s) const { return ldg_w(g[v] + lb + s); }
   __device__ void put(int v, int s, float x) const { g[v][lb + s] = x; }
   __device__ float nbr(int v, unsigned code) const { return ldg_w(g[v] + code); }
   __device__ void put_nbr(int v, unsigned code, float x) const { g[v][code] = x; }
 };
+// Couplings and neighbour codes of node s.
+__device__ __forceinline__ void faces(const LevD<true>& A, int s, bool, float (&c)[6], unsigned (&j)[6]) {
+#pragma unroll
+  for (int f = 0; f < 6; ++f) j[f] = A.nb(f, s);
+#pragma unroll
+  for (int f = 0; f < 6; ++f) c[f] = A.c(f, s, false);
+}
+__device__ __forceinline__ void faces(const LevD<false>& A, int s, bool half, float (&c)[6], unsigned (&j)[6]) {
+  if (A.nd) {
+    const short4 d = A.nd[s];
+    const unsigned i = (unsigned)(A.lb + s);
+    if (half) {
+      const uint4 p = A.pk[s];
+      const unsigned w[3] = {p.x, p.y, p.z};
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const float2 v = __half22float2(*reinterpret_cast<const __half2*>(&w[f]));
+        c[2 * f] = v.x;
+        c[2 * f + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) c[f] = A.pc[f * A.cs + s];
+    }
+    j[0] = c[0] != 0.0f ? i + 1 : i;
+    j[1] = c[1] != 0.0f ? i - 1 : i;
+    j[2] = i + d.x;
+    j[3] = i + d.y;
+    j[4] = i + d.z;
+    j[5] = i + d.w;
+    return;
+  }
+#pragma unroll
+  for (int f = 0; f < 6; ++f) j[f] = A.nb(f, s);
+#pragma unroll
+  for (int f = 0; f < 6; ++f) c[f] = A.c(f, s, half);
+}
 // sum over faces of c (v_i - v_j)
 template <class L> __device__ __forceinline__ float lap_d(const L& A, int vec, int s, float vi, bool half) {
   unsigned j[6];   // loads keep their order: all the codes, then all the values
   float c[6], x[6];
-#pragma unroll
-  for (int f = 0; f < 6; ++f) j[f] = A.nb(f, s);
+  faces(A, s, half, c, j);
 #pragma unroll
   for (int f = 0; f < 6; ++f) x[f] = A.nbr(vec, j[f]);
-#pragma unroll
-  for (int f = 0; f < 6; ++f) c[f] = A.c(f, s, half);
   float a = 0;
 #pragma unroll
   for (int f = 0; f < 6; ++f) a += c[f] * (vi - x[f]);
@@ -884,6 +921,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
       L.n = n;
       L.lb = lb;
       L.c16 = nullptr;
+      L.pk = nullptr;
+      L.nd = nullptr;
       L.g[0] = G.b;
       L.g[1] = G.e;
       L.g[2] = G.o;
@@ -902,6 +941,10 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
         L.pidg = G.idg + lb;
         L.pch = l > 0 ? reinterpret_cast<const unsigned*>(G.child) + lb : nullptr;
         if (l == 0 && mg.c16) L.c16 = mg.c16 + lb;
+        if (l == 0 && v.pk && *v.wide == 0) {
+          L.pk = v.pk + lb;
+          L.nd = v.nd + lb;
+        }
       }
     }
   }
@@ -969,12 +1012,13 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
       reinterpret_cast<unsigned*>(cg_dyn + S.lay.par)[s] = code(lg, mg.L[lg - 1].agg[lb + s], mul);
   }
   // x, r, p, q of the own nodes; the CG operator's couplings
+  // (the FP32 form's r is the V-cycle's right-hand side b)
   T *X = v.x + base, *R = v.r + base, *P = v.p + base, *Q = v.q + base;
   if constexpr (CL) {
     X = reinterpret_cast<T*>(cg_dyn + S.lay.cgv);
-    R = X + na0;
-    P = R + na0;
+    P = X + na0;
     Q = P + na0;
+    R = sizeof(T) == 4 ? reinterpret_cast<T*>(cg_dyn + S.lay.vec[0]) : Q + na0;
   }
   const T* cA = nullptr;   // FP64 form only; the FP32 form reads the level's own couplings
   int csA = 0;
@@ -1057,7 +1101,6 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
       bb = bb + b * b;
       rr = rr + W(r) * W(r);
       if constexpr (sizeof(T) == 4) {
-        L0.put(V_B, i, r);
         L0.put(V_E, i, w1 * L0.idg(i) * r);
       }
     }
@@ -1133,13 +1176,22 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
             const T u = (T)L0.own(V_O, i);
             unsigned j[6];
             float x[6];
-#pragma unroll
-            for (int f = 0; f < 6; ++f) j[f] = L0.nb(f, i);
-#pragma unroll
-            for (int f = 0; f < 6; ++f) x[f] = L0.nbr(V_O, j[f]);
             T w = 0;
+            if constexpr (sizeof(T) == 4) {
+              float cf[6];
+              faces(L0, i, false, cf, j);
 #pragma unroll
-            for (int f = 0; f < 6; ++f) w += cop(f, i) * (u - (T)x[f]);
+              for (int f = 0; f < 6; ++f) x[f] = L0.nbr(V_O, j[f]);
+#pragma unroll
+              for (int f = 0; f < 6; ++f) w += cf[f] * (u - x[f]);
+            } else {
+#pragma unroll
+              for (int f = 0; f < 6; ++f) j[f] = L0.nb(f, i);
+#pragma unroll
+              for (int f = 0; f < 6; ++f) x[f] = L0.nbr(V_O, j[f]);
+#pragma unroll
+              for (int f = 0; f < 6; ++f) w += cA[f * csA + i] * (u - (T)x[f]);
+            }
             return make_uw(u, w);
           },
           [&] {
@@ -1181,7 +1233,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
             R[i] = t.q;
             rn += t.q * t.q;
             const float b = sizeof(T) == 4 ? (float)t.q : (float)(t.q * sc);
-            L0.put(V_B, i, b);
+            if constexpr (sizeof(T) == 8) L0.put(V_B, i, b);
             L0.put(V_E, i, w1 * t.d * b);
           });
       A.post(W(rn), A_RR, nact);

@@ -948,6 +948,13 @@ template <typename T> struct CGVec {
   __half* c16;            // the same in FP16 for the multigrid sweeps (FP32 storage only, else null)
   int* nb;                // compact index of the face neighbour (i itself when absent)
   int cap;
+  // large FP32 bands, whose matrix is read from memory in every sweep: the FP16 couplings with the
+  // inverse diagonal (16 B) and the y and z neighbours as 16-bit offsets (8 B), instead of 12 + 4
+  // and 24 B in 13 loads; *wide is set where an offset does not fit or an x neighbour is not next
+  // in the list (a band across the periodic boundary), and the full lists are read.  Null: not kept.
+  uint4* pk;
+  short4* nd;
+  int* wide;
   T csc;                  // FP64 storage: a power of two near h^2, which takes c32 to order one
 };
 
@@ -965,6 +972,8 @@ __global__ void k_cg_setup(Geo g, ModelC<T> mc, const int* __restrict__ idx, con
     const int q[6] = {n.xp, n.xm, n.yp, n.ym, n.zp, n.zm};
     const T gc = G[p];
     float d = 0;
+    int off[6];
+    __half hc[6];
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
       T c = 0;
@@ -978,9 +987,25 @@ __global__ void k_cg_setup(Geo g, ModelC<T> mc, const int* __restrict__ idx, con
       if (sizeof(T) == 8) v.c32[f * v.cap + i] = cf;
       if (v.c16) v.c16[f * v.cap + i] = __float2half_rn(cf);
       v.nb[f * v.cap + i] = j;
+      off[f] = j - i;
+      hc[f] = __float2half_rn(cf);
       d += cf;
     }
-    v.idg[i] = d > 0.0f ? 1.0f / d : 1.0f;
+    const float di = d > 0.0f ? 1.0f / d : 1.0f;
+    v.idg[i] = di;
+    if (v.pk) {
+      uint4 p;
+      unsigned* w = reinterpret_cast<unsigned*>(&p);
+#pragma unroll
+      for (int f = 0; f < 3; ++f) w[f] = __half_as_ushort(hc[2 * f]) | ((unsigned)__half_as_ushort(hc[2 * f + 1]) << 16);
+      w[3] = __float_as_uint(di);
+      v.pk[i] = p;
+      v.nd[i] = make_short4((short)off[2], (short)off[3], (short)off[4], (short)off[5]);
+      bool fits = (off[0] == 0 || off[0] == 1) && (off[1] == 0 || off[1] == -1);
+#pragma unroll
+      for (int f = 2; f < 6; ++f) fits = fits && off[f] == (int)(short)off[f];
+      if (!fits) *v.wide = 1;
+    }
   }
 }
 

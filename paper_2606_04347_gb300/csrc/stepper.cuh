@@ -330,7 +330,7 @@ template <typename T> class Stepper : public PlanBase {
     sS_ = alloc<C>(g_.nhat);
     sSu_ = alloc<C>(g_.nhat);
     T** reals[] = {&phiA_, &phiB_, &phit_, &lap_, &gx_, &gy_, &gz_, &rr_, &wm_, &r2_, &ut_, &G_, &w_,
-                   &cg_.x, &cg_.r, &cg_.p, &cg_.q};
+                   &cg_.x, &cg_.p, &cg_.q};
     for (T** r : reals) *r = alloc<T>(g_.n);
     for (T** r : reals) ETD_CUDA(cudaMemset(*r, 0, sizeof(T) * g_.n));
     cg_.cap = (int)g_.n;
@@ -343,6 +343,11 @@ template <typename T> class Stepper : public PlanBase {
       // couplings are sums of g / h^2 with g of order one: a power of two near the smallest h^2
       const double hm = std::min(std::min(g_.hx, g_.hy), g_.dim == 2 ? g_.hx : g_.hz);
       cg_.csc = sizeof(T) == 4 ? (T)1 : (T)std::ldexp(1.0, 2 * std::ilogb(hm));
+    }
+    if (sizeof(T) == 4 && g_.n > kCgPackedGrid) {
+      cg_.pk = alloc<uint4>(g_.n);
+      cg_.nd = alloc<short4>(g_.n);
+      cg_.wide = alloc<int>(1);
     }
     float** fl[] = {&cg_.b, &cg_.e, &cg_.o, &cg_.t, &cg_.idg};
     for (float** f : fl) {
@@ -362,6 +367,9 @@ template <typename T> class Stepper : public PlanBase {
       h = alloc<T>(g_.n);
       ETD_CUDA(cudaMemset(h, 0, sizeof(T) * g_.n));
     }
+    // FP32: the residual is the V-cycle's right-hand side
+    if constexpr (sizeof(T) == 4) cg_.r = cg_.b;
+    else cg_.r = alloc<T>(g_.n);
     init_multigrid();
     cg_prepare();
     mask_ = alloc<unsigned char>(g_.n);
@@ -756,6 +764,7 @@ template <typename T> class Stepper : public PlanBase {
 
   void cg_setup(const T* G) {
     CGVec<T> v = cg_;
+    if (v.wide) ETD_CUDA(cudaMemsetAsync(v.wide, 0, sizeof(int), st_));
     timed(ETD_K_BAND, 0.0,
           [&] { k_cg_setup<T><<<nsm_ * 8, 256, 0, st_>>>(g_, mc_, idx_, count_, mask_, bmap_, G, v, ncomp_); });
     mg_setup();
@@ -1647,6 +1656,7 @@ template <typename T> class Stepper : public PlanBase {
   // batch, whose solves run on fewer blocks anyway, up to twice that (8 runs: 18.7 against 17.4 ms).
   static constexpr int kCgPerBlock = sizeof(T) == 4 ? 1024 : 512, kCgPerCluster = sizeof(T) == 4 ? 256 : 64;
   static constexpr long long kCgClusterGrid = 1LL << 19, kCgHybridGrid = 1LL << 20;
+  static constexpr long long kCgPackedGrid = 1LL << 21;   // larger grids: bands whose matrix does not fit shared memory
   static constexpr int kCgHybridMax = 112 * 1024;
   int cg_engine_ = 0, cg_blocks_ = 0;        // frozen band: engine (1 + CG_*) and blocks; 0: unknown
   bool cluster_ok_ = true;

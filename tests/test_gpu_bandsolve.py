@@ -29,7 +29,11 @@ def _params(n, prec):
 def _membrane(p, kind, rng):
     if kind == "full":      # every point in the band, g between 0.46 and 1.125
         return rng.uniform(0.2, 0.8, size=p.shape)
-    r = np.sqrt(sum(c ** 2 for c in wl.grid(p.n, p.half_len, p.dim)))
+    ax = wl.grid(p.n, p.half_len, p.dim)
+    if kind == "corner":    # a sphere around the box's corner: the band crosses every boundary
+        r = np.sqrt(sum((np.pi - np.abs(c)) ** 2 for c in ax))
+        return wl.tanh_profile(1.6 - r, 0.09) * np.ones(p.shape)
+    r = np.sqrt(sum(c ** 2 for c in ax))
     eps = {"shell": 0.25, "thin": 0.09}[kind]
     return wl.tanh_profile(1.6 - r, eps) * np.ones(p.shape)
 
@@ -60,9 +64,11 @@ def test_band_solve_sizes_match_oracle(n, kind, prec):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
-@pytest.mark.parametrize("n,kind", [((128, 128, 64), "thin"), ((128, 128, 128), "shell"), ((256, 64, 64), "thin")])
+@pytest.mark.parametrize("n,kind", [((128, 128, 64), "thin"), ((128, 128, 128), "shell"), ((256, 64, 64), "thin"),
+                                    ((256, 128, 128), "shell"), ((256, 128, 128), "corner"), ((64, 64, 64), "corner")])
 def test_large_band_solve_residual(n, kind, prec):
-    """Bands past one cluster, of a size the host does not know (the hybrid or the grid engine):
+    """Bands past one cluster, of a size the host does not know (the hybrid or the grid engine; the
+    largest with the packed matrix, and across the periodic boundary, where it does not apply):
     the solution's own residual, formed by the oracle's operator, and its mean.  FP32: rounding w
     to FP32 alone leaves a residual of eps32 max(diag) |w| / |b|, below 1e-3 here."""
     p = _params(n, prec)
