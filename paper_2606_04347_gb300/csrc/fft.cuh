@@ -119,6 +119,13 @@ __host__ __device__ __forceinline__ int pitch_b(int nz) {
 }
 
 
+// Extra elements between the planes of a pass-A tile.  The column stages read and write ZB planes
+// side by side (consecutive lanes: plane, then kx), and a plane of 16 rows is a multiple of 128
+// bytes whatever the row pitch: without the skew the planes of one kx share their banks (a
+// ZB-way conflict on every column access; 256^3 FP32, ZB = 4: a launch 48 -> 44 us).
+__host__ __device__ __forceinline__ int plane_skew(int zb, int csize) { return zb > 1 ? 128 / csize / zb : 0; }
+
+
 // Tile choice shared by the plan and the allocation-free entry point.  Returns false if the
 // grid is not supported.  smemA: pass-A tile; smemB1: one pass-B operand tile.
 //   pass A: ZB z-planes x Y2 rows per CTA; zb_req > 0 asks for ZB (a divisor of Nz), else
@@ -142,7 +149,7 @@ inline bool choose_tiles(Geo& g, size_t csize, size_t& smemA, size_t& smemB1, in
   g.ZB = g.nz == 1 ? 1 : (g.nz < zb ? g.nz : zb);
   if (g.nz % g.ZB) return false;
   const int rsa = pitch_a(g.nx);
-  smemA = (size_t)g.ZB * g.Y2 * rsa * csize;
+  smemA = (size_t)g.ZB * (g.Y2 * rsa + plane_skew(g.ZB, (int)csize)) * csize;
   const int rsb = pitch_b(g.nz);
   const int kbmax = passb_max_rows(g.nz) / g.Y1;
   if (kb_req > 0) {
@@ -409,7 +416,8 @@ template <typename C> struct OutP {
 };
 
 // ---- pass A: x real-to-complex + inner y DFT ------------------------------------------
-// Tile: rows r = zz * Y2 + j (plane z0 + zz, y = n1 + Y1 j), row stride pad16(nxh-1)+1.
+// Tile: rows r = zz * Y2 + j (plane z0 + zz, y = n1 + Y1 j), row stride pad16(nxh-1)+1, planes
+// plane_skew elements apart.
 
 template <typename T, typename Pro, int R, int S>
 __device__ __forceinline__ void passA_rows_fwd(const Geo& g, const Pro& pro, typename Cplx<T>::type* tile, int rs,
@@ -434,7 +442,7 @@ __device__ __forceinline__ void passA_rows_fwd(const Geo& g, const Pro& pro, typ
       v[j] = ok ? C{pro(i0 + x), pro(i1 + x)} : C{0, 0};
     }
     // the row pair's two tile rows (2 rs >= S (R + 1) values) double as the exchange scratch
-    C* row = tile + (ok ? r0 : 0) * rs;
+    C* row = tile + (ok ? r0 * rs + (r0 >> ly) * plane_skew(g.ZB, sizeof(C)) : 0);
     team_fft<C, R, S, false>(v, t, row, twx, ok);
     __syncwarp();
     // unpack the two real rows, A[k] = (Z[k] + conj Z[N-k])/2, B[k] = (Z[k] - conj Z[N-k])/(2i),
@@ -467,12 +475,13 @@ __device__ __forceinline__ void passA_cols_fwd(const Geo& g, const typename Cplx
                                                int n1, typename Cplx<T>::type* __restrict__ out,
                                                const typename Cplx<T>::type* __restrict__ twy) {
   using C = typename Cplx<T>::type;
+  const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
   const int ncols = g.ZB * g.nxh;
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
     const int zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
     C v[Y > 1 ? Y : 1];
 #pragma unroll
-    for (int j = 0; j < Y; ++j) v[j] = tile[(zz * Y + j) * rs + pad16(kx)];
+    for (int j = 0; j < Y; ++j) v[j] = tile[zz * pp + j * rs + pad16(kx)];
     dftN<C, Y, false>(v);
 #pragma unroll
     for (int k2 = 0; k2 < Y; ++k2) {
@@ -546,13 +555,14 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
                                                       const typename Cplx<T>::type* __restrict__ twy) {
   using C = typename Cplx<T>::type;
   C* stg = tile;
+  const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
   const int ncols = g.ZB * g.nxh, nt = blockDim.x, t = threadIdx.x;
   const int nmain = ncols < nt ? ncols : nt, ntail = ncols - nmain;
   C v[Y > 1 ? Y : 1];
   if (t < ntail) {
     const int col = nmain + t, zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
 #pragma unroll
-    for (int j = 0; j < Y; ++j) v[j] = tile[(zz * Y + j) * rs + pad16(kx)];
+    for (int j = 0; j < Y; ++j) v[j] = tile[zz * pp + j * rs + pad16(kx)];
     dftN<C, Y, false>(v);
 #pragma unroll
     for (int k2 = 0; k2 < Y; ++k2) side[t * Y + k2] = (n1 && k2) ? cmul(v[k2], ldg_c(&twy[n1 * k2])) : v[k2];
@@ -561,7 +571,7 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
   const int zz = t & (g.ZB - 1), kx = t >> log2_of(g.ZB);
   if (mine) {
 #pragma unroll
-    for (int j = 0; j < Y; ++j) v[j] = tile[(zz * Y + j) * rs + pad16(kx)];
+    for (int j = 0; j < Y; ++j) v[j] = tile[zz * pp + j * rs + pad16(kx)];
   }
   __syncthreads();
   if (mine) {
@@ -630,6 +640,7 @@ __device__ __forceinline__ void passA_cols_inv(const Geo& g, typename Cplx<T>::t
                                                const typename Cplx<T>::type* __restrict__ in,
                                                const typename Cplx<T>::type* __restrict__ twy) {
   using C = typename Cplx<T>::type;
+  const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
   const int ncols = g.ZB * g.nxh;
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
     const int zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
@@ -642,7 +653,7 @@ __device__ __forceinline__ void passA_cols_inv(const Geo& g, typename Cplx<T>::t
     }
     dftN<C, Y, true>(v);
 #pragma unroll
-    for (int j = 0; j < Y; ++j) tile[(zz * Y + j) * rs + pad16(kx)] = v[j];
+    for (int j = 0; j < Y; ++j) tile[zz * pp + j * rs + pad16(kx)] = v[j];
   }
 }
 
@@ -654,6 +665,7 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
                                                       const typename Cplx<T>::type* __restrict__ twy) {
   using C = typename Cplx<T>::type;
   const C* stg = tile;
+  const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
   const int ncols = g.ZB * g.nxh, nt = blockDim.x, t = threadIdx.x;
   const int nmain = ncols < nt ? ncols : nt, ntail = ncols - nmain;
   C v[Y > 1 ? Y : 1];
@@ -675,21 +687,21 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
     }
     dftN<C, Y, true>(v);
 #pragma unroll
-    for (int j = 0; j < Y; ++j) tile[(zz * Y + j) * rs + pad16(kx)] = v[j];
+    for (int j = 0; j < Y; ++j) tile[zz * pp + j * rs + pad16(kx)] = v[j];
   }
   if (ntail > 0) {
     if (tl) {
       if (n1) xt = cmulc(xt, ldg_c(&twy[n1 * tk2]));
-      tile[((tcol & (g.ZB - 1)) * Y + tk2) * rs + pad16(tcol >> log2_of(g.ZB))] = xt;
+      tile[(tcol & (g.ZB - 1)) * pp + tk2 * rs + pad16(tcol >> log2_of(g.ZB))] = xt;
     }
     __syncthreads();
     if (t < ntail) {
       const int col = nmain + t, z2 = col & (g.ZB - 1), k = col >> log2_of(g.ZB);
 #pragma unroll
-      for (int k2 = 0; k2 < Y; ++k2) v[k2] = tile[(z2 * Y + k2) * rs + pad16(k)];
+      for (int k2 = 0; k2 < Y; ++k2) v[k2] = tile[z2 * pp + k2 * rs + pad16(k)];
       dftN<C, Y, true>(v);
 #pragma unroll
-      for (int j = 0; j < Y; ++j) tile[(z2 * Y + j) * rs + pad16(k)] = v[j];
+      for (int j = 0; j < Y; ++j) tile[z2 * pp + j * rs + pad16(k)] = v[j];
     }
   }
 }
@@ -709,7 +721,7 @@ __device__ __forceinline__ void passA_rows_inv(const Geo& g, const Epi& epi, typ
     const int r0 = 2 * q;
     const long long i0 = ((long long)(z0 + (r0 >> ly)) * g.ny + n1 + g.Y1 * (r0 & (g.Y2 - 1))) * N;
     const long long i1 = i0 + (long long)g.Y1 * N;
-    C* ra = tile + (ok ? r0 : 0) * rs;
+    C* ra = tile + (ok ? r0 * rs + (r0 >> ly) * plane_skew(g.ZB, sizeof(C)) : 0);
     const C* rb = ra + rs;
     C v[R];
 #pragma unroll
