@@ -829,7 +829,8 @@ __global__ void __launch_bounds__(ETD_PASSA_THREADS, sizeof(T) == 4 ? ETD_PASSA_
 // Tile rows are (kxl, k1) pairs (row index kxl * Y1 + k1) of Nz values, row stride
 // pad16(Nz-1)+1.  Op supplies NI (intermediates transformed forward, 0..2),
 // combine(e, global index, wave, s0, s1) on the spectra (base left in s0) and nout
-// outputs out(o, base, wave), each inverse-transformed into outs.p[o].
+// outputs out(o, base, wave) (kRow: row(o, base, v, row's wave, lane) for a lane's values at once),
+// each inverse-transformed into outs.p[o].
 
 template <typename T, int Y, bool INV>
 __device__ __forceinline__ void passB_cols(const Geo& g, int kbn, const typename Cplx<T>::type* src,
@@ -961,8 +962,12 @@ __device__ __forceinline__ void passB_rows(const Geo& g, const Op& op, int kx0, 
       C v[R];
       const int kxl = ok ? row / g.Y1 : 0, k1 = ok ? row - kxl * g.Y1 : 0;
       const Wave wr = make_wave_row(g, kx0 + kxl, k2 + g.Y2 * k1);
+      if constexpr (Op::kRow) {
+        op.template row<R, S>(o, base[rr], v, wr, t);
+      } else {
 #pragma unroll
-      for (int k = 0; k < R; ++k) v[k] = ok ? op.out(o, base[rr][k], make_wave_z<N>(wr, t + S * k)) : C{0, 0};
+        for (int k = 0; k < R; ++k) v[k] = ok ? op.out(o, base[rr][k], make_wave_z<N>(wr, t + S * k)) : C{0, 0};
+      }
       C* r0 = tb + (ok ? row : 0) * rs;
       team_fft<C, R, S, true>(v, t, r0, twz, ok);
       __syncwarp();

@@ -47,14 +47,37 @@ __device__ __forceinline__ Row3<double> load_row(const double* t, int m) {
 // The whole FP32 row: phi0 (high part), tau phi1, tau phi2, phi0 (low part).
 __device__ __forceinline__ float4 load_row4(const float* t, int m) { return __ldg(reinterpret_cast<const float4*>(t) + m); }
 
-template <typename T, typename C>
-__device__ __forceinline__ C deriv_mult(int o, C v, const Wave& w, const SpecConst<T>& k) {
-  // o = 0: identity, 1: Laplacian (lambda), 2..4: d/dx, d/dy, d/dz (i k, Nyquist -> 0)
-  if (o == 0) return cscale(v, k.inv_n);
-  if (o == 1) return cscale(v, -k.ksq * (T)w.m * k.inv_n);
-  const int s = (o == 2) ? w.sx : (o == 3 ? w.sy : w.sz);
-  const T f = k.kscale * (T)s * k.inv_n;
-  return C{-f * v.y, f * v.x};
+// Multipliers of the R values (kz = t + S r) that a lane of a row holds, by code: 0 identity, 1
+// Laplacian (lambda), 2..4 d/dx, d/dy, d/dz (i k, Nyquist -> 0).  The multiplier is chosen once, its x and y parts are the row's, and kz and |k|^2 are formed in T (integers below 2^24:
+// exact) instead of by a conversion per element and output.
+template <typename T, int R, int S, typename C>
+__device__ __forceinline__ void deriv_row(int code, const C (&base)[R], C (&v)[R], const Wave& w, int t,
+                                          const SpecConst<T>& k) {
+  constexpr int N = R * S, h = N / 2;
+  const T tz = (T)t;
+  if (code == 0) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = cscale(base[r], k.inv_n);
+  } else if (code == 1) {
+    const T mr = (T)w.m;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const T fz = N == 1 || S * r < h ? tz + (T)(S * r) : (T)(N - S * r) - tz;   // |kz|
+      v[r] = cscale(base[r], -k.ksq * (mr + fz * fz) * k.inv_n);
+    }
+  } else if (code == 4) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      // signed kz, 0 at the Nyquist index
+      const T sz = S * r < h ? tz + (T)(S * r) : (S * r == h && t == 0 ? (T)0 : tz + (T)(S * r - N));
+      const T f = k.kscale * sz * k.inv_n;
+      v[r] = C{-f * base[r].y, f * base[r].x};
+    }
+  } else {
+    const T f = k.kscale * (T)(code == 2 ? w.sx : w.sy) * k.inv_n;
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = C{-f * base[r].y, f * base[r].x};
+  }
 }
 
 // Forward only: store the spectrum (plan layout).
@@ -63,6 +86,7 @@ template <typename T> struct OpStore {
   __device__ const void* pre() const { return nullptr; }
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 1;
+  static constexpr bool kRow = false;
   int nout;
   C* spec;
   __device__ void combine(int, long long ge, const Wave&, C& s0, C&) const { spec[ge] = s0; }
@@ -70,18 +94,22 @@ template <typename T> struct OpStore {
 };
 
 // Load a stored spectrum and emit multipliers of it (identity, Laplacian, gradient).
-// `sel` lists the outputs (codes of deriv_mult).
+// `sel` lists the outputs (codes of deriv_row).
 template <typename T, typename S = typename Cplx<T>::type> struct OpDeriv {
   using C = typename Cplx<T>::type;
   __device__ const void* pre() const { return nullptr; }
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 0;
+  static constexpr bool kRow = true;
   int nout;
   int sel[5];
   const S* spec;
   SpecConst<T> k;
   __device__ void combine(int, long long ge, const Wave&, C& s0, C&) const { s0 = conv<C>(spec[ge]); }
-  __device__ C out(int o, C v, const Wave& w) const { return deriv_mult<T>(sel[o], v, w, k); }
+  template <int NR, int NS>
+  __device__ void row(int o, const C (&base)[NR], C (&v)[NR], const Wave& w, int t) const {
+    deriv_row<T, NR, NS>(sel[o], base, v, w, t, k);
+  }
 };
 
 // phi-stage predictor (Sec. 3.3): R1^ = FFT(R_rest) + kappa/(mu eps^2) lambda FFT(W'-A1 phi),
@@ -92,6 +120,7 @@ template <typename T> struct OpPhiPred {
   __device__ const void* pre() const { return spec_phi; }  // stored spectrum read in combine
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 2;
+  static constexpr bool kRow = true;
   int nout;
   int sel[5];
   C* spec_phi;     // phi^n^ (ETD1: overwritten with phi^{n+1}^)
@@ -114,7 +143,10 @@ template <typename T> struct OpPhiPred {
     }
     s0 = pt;
   }
-  __device__ C out(int o, C v, const Wave& w) const { return deriv_mult<T>(sel[o], v, w, k); }
+  template <int NR, int NS>
+  __device__ void row(int o, const C (&base)[NR], C (&v)[NR], const Wave& w, int t) const {
+    deriv_row<T, NR, NS>(sel[o], base, v, w, t, k);
+  }
 };
 
 // phi-stage corrector: phi^{n+1}^ = S + tau phi2 R1(phi~)^ ; stored and emitted.
@@ -123,6 +155,7 @@ template <typename T> struct OpPhiCorr {
   __device__ const void* pre() const { return spec_S; }  // stored spectrum read in combine
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 2;
+  static constexpr bool kRow = false;
   int nout;
   C* spec_phi;
   const C* spec_S;
@@ -150,6 +183,7 @@ struct OpPhiPredInc {
   __device__ const void* pre() const { return spec_phi; }  // stored spectrum read in combine
   __device__ size_t pre_elem() const { return sizeof(dcomplex); }
   static constexpr int NI = 2;
+  static constexpr bool kRow = true;
   int nout;
   int sel[5];
   dcomplex* spec_phi;
@@ -172,7 +206,10 @@ struct OpPhiPredInc {
       s0 = d1;
     }
   }
-  __device__ C out(int o, C v, const Wave& w) const { return deriv_mult<float>(sel[o], v, w, k); }
+  template <int NR, int NS>
+  __device__ void row(int o, const C (&base)[NR], C (&v)[NR], const Wave& w, int t) const {
+    deriv_row<float, NR, NS>(sel[o], base, v, w, t, k);
+  }
 };
 
 // phi-stage corrector on the double-float spectrum: D = S' + tau phi2 R1(phi~)^ is
@@ -182,6 +219,7 @@ struct OpPhiCorrInc {
   __device__ const void* pre() const { return spec_phi; }  // stored spectrum read in combine
   __device__ size_t pre_elem() const { return sizeof(dcomplex); }
   static constexpr int NI = 2;
+  static constexpr bool kRow = false;
   int nout;
   dcomplex* spec_phi;
   const C* spec_S;
@@ -207,6 +245,7 @@ template <typename T> struct OpUPred {
   __device__ const void* pre() const { return nullptr; }
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 2;
+  static constexpr bool kRow = false;
   int nout;
   C* spec_S;
   int rk2;
@@ -226,6 +265,7 @@ template <typename T> struct OpUCorr {
   __device__ const void* pre() const { return spec_S; }  // stored spectrum read in combine
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 1;
+  static constexpr bool kRow = false;
   int nout;
   const C* spec_S;
   SpecConst<T> k;
@@ -243,6 +283,7 @@ template <typename T> struct OpToStd {
   __device__ const void* pre() const { return nullptr; }
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 1;
+  static constexpr bool kRow = false;
   int nout;
   C* dst;
   int ny, nxh;
@@ -257,6 +298,7 @@ template <typename T> struct OpFromStd {
   __device__ const void* pre() const { return nullptr; }
   __device__ size_t pre_elem() const { return sizeof(C); }
   static constexpr int NI = 0;
+  static constexpr bool kRow = false;
   int nout;
   const C* src;
   int ny, nxh;
