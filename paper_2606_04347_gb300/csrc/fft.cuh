@@ -981,8 +981,13 @@ __device__ __forceinline__ void passB_rows(const Geo& g, const Op& op, int kx0, 
   }
 }
 
+// FP32 CTAs per SM that the registers are sized for: the one-input operators fit three (80
+// registers, 56 bytes spilled; 256^3 U corrector 77 -> 73 us); the derivatives of a stored spectrum,
+// which hold it across four outputs, and the two-input ones lose by it (111 -> 118 us).
+constexpr int passb_minb(int ni, int fam) { return ni == 1 && fam == 0 ? 3 : ETD_PASSB_MINB; }
+
 template <typename T, typename Op, int FAM = 0>
-__global__ void __launch_bounds__(ETD_PASSB_THREADS, sizeof(T) == 4 ? ETD_PASSB_MINB : 1) passB(Geo g, Op op, const typename Cplx<T>::type* __restrict__ in0,
+__global__ void __launch_bounds__(ETD_PASSB_THREADS, sizeof(T) == 4 ? passb_minb(Op::NI, FAM) : 1) passB(Geo g, Op op, const typename Cplx<T>::type* __restrict__ in0,
                                              const typename Cplx<T>::type* __restrict__ in1,
                                              OutP<typename Cplx<T>::type> outs,
                                              const typename Cplx<T>::type* __restrict__ twy,
