@@ -27,6 +27,7 @@
 #include <cuda.h>  // CUtensorMap (type only; the plan encodes maps through the runtime's driver entry point)
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <type_traits>
 #include "df32.cuh"
 
 namespace etd {
@@ -470,13 +471,70 @@ __device__ __forceinline__ void passA_rows_fwd(const Geo& g, const Pro& pro, typ
   }
 }
 
+// 16-point DFT of a column held by 4 lanes (rank q of 4) with 4 values each, element q + 4 r in v[r]
+// on entry and on exit: DFT4 over r, the twiddle w_16^(q k), a 4 x 4 transpose over the lanes, DFT4.
+// tw: w_N^e with N = 16 st.
+template <typename C, bool INV>
+__device__ __forceinline__ void dft16_quad(C (&v)[4], int q, const C* __restrict__ tw, int st) {
+  dft4<C, INV>(v);
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    const C w = ldg_c(&tw[st * q * k]);
+    v[k] = INV ? cmulc(v[k], w) : cmul(v[k], w);
+  }
+  C u[4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {   // lane q sends v[q ^ s] to lane q ^ s and takes its v[q]
+    const int i = q ^ s;
+    const C x = i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3]));
+    const C y{__shfl_xor_sync(0xffffffffu, x.x, s), __shfl_xor_sync(0xffffffffu, x.y, s)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i == k) u[k] = y;
+  }
+  dft4<C, INV>(u);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = u[k];
+}
+// FP64: the columns beyond whole warps of a 16-row tile go to the next warp, four lanes each.  A
+// warp's column stage costs its FP64 instructions (224 at 64 clocks) however few lanes have a
+// column, and 130 columns (128^3, two planes) are four warps and two lanes: the sub-partition with
+// the fifth warp had twice the work of the others (128^3: a launch 119 -> 113 us).
+template <typename T> __device__ __forceinline__ bool quad_tail(int ncols, int Y) {
+  return std::is_same<T, double>::value && Y == 16 && ncols >= 32 && (ncols & 31) > 0 && (ncols & 31) <= 8 &&
+         (ncols | 31) < ETD_PASSA_THREADS;
+}
+
 template <typename T, int Y>
 __device__ __forceinline__ void passA_cols_fwd(const Geo& g, const typename Cplx<T>::type* tile, int rs, int z0,
                                                int n1, typename Cplx<T>::type* __restrict__ out,
                                                const typename Cplx<T>::type* __restrict__ twy) {
   using C = typename Cplx<T>::type;
   const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
-  const int ncols = g.ZB * g.nxh;
+  const int all = g.ZB * g.nxh;
+  const bool quad = quad_tail<T>(all, Y);
+  const int ncols = quad ? all & ~31 : all;
+  if constexpr (std::is_same<T, double>::value && Y == 16) {
+    const int q0 = (int)threadIdx.x - ncols;
+    if (quad && q0 >= 0 && q0 < 32) {
+      const int col = ncols + (q0 >> 2), q = q0 & 3, zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
+      C v[4] = {};
+      if (col < all) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = tile[zz * pp + (q + 4 * r) * rs + pad16(kx)];
+      }
+      dft16_quad<C, false>(v, q, twy, g.ny >> 4);
+      if (col < all) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int k2 = q + 4 * r;
+          C x = v[r];
+          if (n1 && k2) x = cmul(x, ldg_c(&twy[n1 * k2]));
+          out[((long long)(k2 * g.nxh + kx) * g.Y1 + n1) * g.nz + z0 + zz] = x;
+        }
+      }
+    }
+  }
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
     const int zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
     C v[Y > 1 ? Y : 1];
@@ -557,7 +615,8 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
   C* stg = tile;
   const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
   const int ncols = g.ZB * g.nxh, nt = blockDim.x, t = threadIdx.x;
-  const int nmain = ncols < nt ? ncols : nt, ntail = ncols - nmain;
+  const bool quad = quad_tail<T>(ncols, Y);
+  const int nmain = quad ? ncols & ~31 : (ncols < nt ? ncols : nt), ntail = quad ? 0 : ncols - nmain;
   C v[Y > 1 ? Y : 1];
   if (t < ntail) {
     const int col = nmain + t, zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
@@ -573,7 +632,26 @@ __device__ __forceinline__ void passA_cols_fwd_staged(const Geo& g, typename Cpl
 #pragma unroll
     for (int j = 0; j < Y; ++j) v[j] = tile[zz * pp + j * rs + pad16(kx)];
   }
+  C qv[4] = {};
+  const int qc = (t - nmain) >> 2, qq = t & 3, qz = (nmain + qc) & (g.ZB - 1), qk = (nmain + qc) >> log2_of(g.ZB);
+  const bool qw = quad && t >= nmain && t < nmain + 32, qm = qw && nmain + qc < ncols;
+  if (qm) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) qv[r] = tile[qz * pp + (qq + 4 * r) * rs + pad16(qk)];
+  }
   __syncthreads();
+  if constexpr (std::is_same<T, double>::value && Y == 16) {
+    if (qw) {
+      dft16_quad<C, false>(qv, qq, twy, g.ny >> 4);
+      if (qm) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int k2 = qq + 4 * r;
+          stg[(k2 * g.nxh + qk) * g.ZB + qz] = (n1 && k2) ? cmul(qv[r], ldg_c(&twy[n1 * k2])) : qv[r];
+        }
+      }
+    }
+  }
   if (mine) {
     dftN<C, Y, false>(v);
 #pragma unroll
@@ -641,7 +719,30 @@ __device__ __forceinline__ void passA_cols_inv(const Geo& g, typename Cplx<T>::t
                                                const typename Cplx<T>::type* __restrict__ twy) {
   using C = typename Cplx<T>::type;
   const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
-  const int ncols = g.ZB * g.nxh;
+  const int all = g.ZB * g.nxh;
+  const bool quad = quad_tail<T>(all, Y);
+  const int ncols = quad ? all & ~31 : all;
+  if constexpr (std::is_same<T, double>::value && Y == 16) {
+    const int q0 = (int)threadIdx.x - ncols;
+    if (quad && q0 >= 0 && q0 < 32) {
+      const int col = ncols + (q0 >> 2), q = q0 & 3, zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
+      C v[4] = {};
+      if (col < all) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int k2 = q + 4 * r;
+          C x = in[((long long)(k2 * g.nxh + kx) * g.Y1 + n1) * g.nz + z0 + zz];
+          if (n1 && k2) x = cmulc(x, ldg_c(&twy[n1 * k2]));
+          v[r] = x;
+        }
+      }
+      dft16_quad<C, true>(v, q, twy, g.ny >> 4);
+      if (col < all) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) tile[zz * pp + (q + 4 * r) * rs + pad16(kx)] = v[r];
+      }
+    }
+  }
   for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
     const int zz = col & (g.ZB - 1), kx = col >> log2_of(g.ZB);
     C v[Y > 1 ? Y : 1];
@@ -667,7 +768,8 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
   const C* stg = tile;
   const int pp = Y * rs + plane_skew(g.ZB, sizeof(C));   // plane pitch
   const int ncols = g.ZB * g.nxh, nt = blockDim.x, t = threadIdx.x;
-  const int nmain = ncols < nt ? ncols : nt, ntail = ncols - nmain;
+  const bool quad = quad_tail<T>(ncols, Y);
+  const int nmain = quad ? ncols & ~31 : (ncols < nt ? ncols : nt), ntail = quad ? 0 : ncols - nmain;
   C v[Y > 1 ? Y : 1];
   const bool mine = t < nmain;
   const int zz = t & (g.ZB - 1), kx = t >> log2_of(g.ZB);
@@ -679,7 +781,28 @@ __device__ __forceinline__ void passA_cols_inv_staged(const Geo& g, typename Cpl
   const int tcol = nmain + t / Y, tk2 = t % Y;
   C xt = C{0, 0};
   if (tl) xt = stg[(tk2 * g.nxh + (tcol >> log2_of(g.ZB))) * g.ZB + (tcol & (g.ZB - 1))];
+  C qv[4] = {};
+  const int qc = (t - nmain) >> 2, qq = t & 3, qz = (nmain + qc) & (g.ZB - 1), qk = (nmain + qc) >> log2_of(g.ZB);
+  const bool qw = quad && t >= nmain && t < nmain + 32, qm = qw && nmain + qc < ncols;
+  if (qm) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) qv[r] = stg[((qq + 4 * r) * g.nxh + qk) * g.ZB + qz];
+  }
   __syncthreads();
+  if constexpr (std::is_same<T, double>::value && Y == 16) {
+    if (qw) {
+      if (n1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (qq + 4 * r) qv[r] = cmulc(qv[r], ldg_c(&twy[n1 * (qq + 4 * r)]));
+      }
+      dft16_quad<C, true>(qv, qq, twy, g.ny >> 4);
+      if (qm) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) tile[qz * pp + (qq + 4 * r) * rs + pad16(qk)] = qv[r];
+      }
+    }
+  }
   if (mine) {
     if (n1) {
 #pragma unroll
