@@ -17,8 +17,9 @@
  *  - Fields are dense, C-ordered, x fastest: index (k*Ny + j)*Nx + i for 3D, j*Nx + i for
  *    2D.  Grid point (i,j,k) sits at (-X + i*hx, -Y + j*hy, -Z + k*hz), h = 2X/N (Sec. 2.1).
  *  - Element type is double for ETD_FP64 and float for ETD_FP32_MIXED.  FP32_MIXED keeps
- *    the phi-function tables (built in FP64, rounded once), every reduction (mass, volume,
- *    energy, CG dot products) and the scalar constraint terms in FP64.
+ *    the phi-function tables (built in FP64, rounded once) and the scalar constraint terms in
+ *    FP64, and every reduction (mass, volume, energy, CG dot products) in double-float (about
+ *    48 bits) within a block, in FP64 across the mass, volume and energy sums' blocks.
  *  - Field pointers are DEVICE pointers owned by the caller (for example PyTorch tensors
  *    on the plan's device).  They must stay valid until the enqueued work completes.  The
  *    library never frees them.  All work is enqueued on the stream given to etd_plan.
@@ -115,6 +116,8 @@ typedef struct {
  * Every device wait is bounded: a grid barrier of the band solve gives up after
  * ETD_WAIT_BUDGET clock cycles (default 4e9) and a tensor copy of the FFT after
  * ETD_WAIT_TRIES mbarrier polls (default 2^22); both environment variables are read here.
+ * (A solve inside one thread-block cluster waits at the hardware's cluster barrier, which does
+ * not spin; it gives up only for a budget below zero.)
  * A wait that gives up makes the call that observes it return ETD_ETIMEOUT, the device
  * context stays usable (the waiting blocks return, a block whose copy is late waits for it
  * once more before it leaves). */

@@ -1406,7 +1406,7 @@ template <typename T> class Stepper : public PlanBase {
     auto k = k_lanczos<T>;
     // Nodes spread over all SMs before they fill blocks: the FP64 work of a node on 2 operations a
     // clock and SM, and block sums over as few warps as hold nodes (5852 nodes FP64, 8 steps: 3
-    // blocks of 1024 184 us, 46 of 128 58 us; a block's threads a power of two from 128 on).
+    // blocks of 1024 182 us, 46 of 128 62 us; a block's threads a power of two from 128 on).
     int threads = 128;
     while (threads < 1024 && (long long)threads * nsm_ < fixed_count_) threads *= 2;
     const int grid = std::max(1, std::min(nsm_, (fixed_count_ + threads - 1) / threads));

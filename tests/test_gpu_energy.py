@@ -48,3 +48,23 @@ def test_energy_sums_match_oracle(n, kind, prec, tol):
     mb, lo, hi = omodel.bound_stats(u, G, p.recover_delta)
     assert d["band_size"] == band.sum() and (d["max_bound"], d["umin"], d["umax"]) == (mb, lo, hi)
     assert abs(d["volume"] - omodel.volume(phi, p)) <= 1e-13 * phi.sum()
+
+
+def test_step_of_an_unaligned_field():
+    """u one element past a 16-byte boundary: the mass sum takes its one-value loads.  Only the
+    order of that sum differs, so the FP64 results agree to a few roundings of the mass (its
+    relative error is below 1e-14 and the step is Lipschitz in it: 1e-12)."""
+    p = _params((64, 64, 1), 0).replace(scheme=1, tau=1e-3, M=100.0, cg_rtol=1e-13)
+    rng = np.random.default_rng(8)
+    phi = _membrane(p, "shell", rng)
+    u = rng.uniform(0.3, 0.7, size=p.shape)
+    plan = Plan(p)
+    phid, ud = torch.tensor(phi, device=DEV), torch.tensor(u, device=DEV)
+    buf = torch.zeros(u.size + 1, dtype=torch.float64, device=DEV)
+    buf[1:] = ud.reshape(-1)
+    uu = buf[1:].view(u.shape)
+    assert uu.data_ptr() % 16 != 0
+    a = plan.step(phid, ud, 1, diag=True)
+    b = plan.step(phid, uu, 1, diag=True)
+    assert abs(a["mass"] - b["mass"]) <= 1e-13 * abs(a["mass"])
+    assert float((ud - uu).norm()) <= 1e-12 * float(ud.norm())
