@@ -7,6 +7,7 @@
 #include <cstring>
 #include <vector>
 #include "bandcg.cuh"
+#include "fft_std.cuh"
 #include "kernels.cuh"
 #include "krylov.cuh"
 #include "mgsetup.cuh"
@@ -153,14 +154,18 @@ template <typename T> class Stepper : public PlanBase {
 
   void fft_forward(const void* field, void* half) override {
     fwd(ProLoad<T>{static_cast<const T*>(field)}, I_[0]);
-    OpToStd<T> op{0, static_cast<C*>(half), g_.ny, g_.nxh};
-    passb(op, I_[0], nullptr, outs({}));
+    if (!std_pass<false>(I_[0], static_cast<C*>(half), T(1))) {
+      OpToStd<T> op{0, static_cast<C*>(half), g_.ny, g_.nxh};
+      passb(op, I_[0], nullptr, outs({}));
+    }
     sync_check();
   }
 
   void fft_inverse(const void* half, void* field) override {
-    OpFromStd<T> op{1, static_cast<const C*>(half), g_.ny, g_.nxh, sk_.inv_n};
-    passb(op, nullptr, nullptr, outs({I_[0]}));
+    if (!std_pass<true>(static_cast<const C*>(half), I_[0], sk_.inv_n)) {
+      OpFromStd<T> op{1, static_cast<const C*>(half), g_.ny, g_.nxh, sk_.inv_n};
+      passb(op, nullptr, nullptr, outs({I_[0]}));
+    }
     inv(I_[0], EpiStore<T>{static_cast<T*>(field)});
     sync_check();
   }
@@ -709,6 +714,27 @@ template <typename T> class Stepper : public PlanBase {
       k<<<nkb * g_.Y2, ETD_PASSB_THREADS, smemB, st_>>>(g_, op, in0, in1, o, twy_, twz_);
     });
     ETD_CUDA(cudaGetLastError());
+  }
+
+  // Pass B between the intermediate and the standard layout with several kx a CTA; false where
+  // std_blocks keeps passB, or where the plan's pencil count was tuned.
+  template <bool INV> bool std_pass(const C* src, C* dst, T scale) {
+    if constexpr (sizeof(T) != 4) {
+      return false;
+    } else {
+      const int kb = tune_kb_ > 0 ? 0 : std_blocks(g_, sizeof(C), nsm_, INV);
+      if (!kb) return false;
+      Geo g = g_;
+      g.KB = kb;
+      const size_t smem = (size_t)kb * g.Y1 * pitch_b(g.nz) * sizeof(C);
+      auto k = passB_std<T, INV>;
+      set_smem((const void*)k, smem);
+      timed(ETD_K_FFT_B, 2 * spc(), [&] {
+        k<<<(g.nxh + kb - 1) / kb * g.Y2, kStdThreads, smem, st_>>>(g, src, dst, twz_, scale);
+      });
+      ETD_CUDA(cudaGetLastError());
+      return true;
+    }
   }
 
   void set_smem(const void* k, size_t bytes) {

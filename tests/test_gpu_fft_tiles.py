@@ -52,3 +52,19 @@ def test_r1_of_an_unaligned_field_matches_oracle(prec, tol):
     plan.remainder(1, phid, None, uu, out)
     want = omodel.R1(phi, u, p, p.A0)
     assert np.linalg.norm(out.cpu().numpy() - want) < tol * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("n", [(256, 256, 256), (128, 256, 256), (256, 128, 128), (256, 256, 64), (96, 256, 64)])
+def test_large_standard_layout_transforms_match_numpy(n):
+    """FP32 pass B with several kx a CTA on its way to and from the standard layout, with whole
+    and ragged last groups (the bound of the transforms above; the arrays end exactly at the grid)."""
+    p = wl.workload("c2", n=16)[0].replace(dim=3, n=n, model=0, precision=1)
+    plan = Plan(p)
+    f = torch.tensor(wl.random_fields(p.shape, 5, -1.0, 1.0), dtype=plan.dtype, device=DEV)
+    half = torch.zeros(p.shape[:-1] + (n[0] // 2 + 1,), dtype=plan.cdtype, device=DEV)
+    back = torch.zeros_like(f)
+    plan.fft_forward(f, half)
+    plan.fft_inverse(half, back)
+    want = np.fft.rfftn(f.cpu().numpy().astype(np.float64))
+    assert np.linalg.norm(half.cpu().numpy() - want) < 2e-6 * np.linalg.norm(want)
+    assert float((back.double() - f.double()).norm()) < 2e-6 * float(f.double().norm())
