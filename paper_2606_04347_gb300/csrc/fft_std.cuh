@@ -14,10 +14,9 @@ constexpr int kStdThreads = 384;
 // already fill half a sector, and those launches are bound by the FP64 pipe), power-of-two nz of 64
 // or more, a tile of which two CTAs fit an SM while two CTAs for each SM are left.  Per launch,
 // passB -> passB_std:
-//   forward, 3 blocks or more: 256^3 92 -> 72 us, 256x256x128 44.7 -> 34.2 us, 256x128x128 22.3 -> 13.0, 256x256x64
-//     22.2 -> 12.6, 128^3 15.2 -> 11.5, 128x256x256
-//     45 -> 43, 256x128x256 43 either way; two blocks lose
-//     (96x256x256 31.5 -> 39.6);
+//   forward, 3 blocks or more: 256^3 92 -> 72 us, 256x256x128 44.7 -> 34.2, 256x128x128
+//     22.3 -> 13.0, 256x256x64 22.2 -> 12.6, 128^3 15.2 -> 11.5, 128x256x256 45 -> 43, 256x128x256
+//     43 either way; two blocks lose (96x256x256 31.5 -> 39.6);
 //   inverse, 6 or more (a whole sector) in a tile of 64 KB: 256x128x128 19.2 -> 13.2, 256x256x64
 //     19.8 -> 13.0, 256x32x256 10.8 -> 8.9; beyond, it loses (128^3, 3 blocks: 11.0 -> 12.4;
 //     256x128x256, 104 KB: 34.4 -> 45.9; what holds the large tiles' loads up was not found).
