@@ -461,6 +461,11 @@ template <typename Load, typename Store> __device__ __forceinline__ void nodes(i
   nodes(n, load, [] {}, store);
 }
 
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <typename T, int MODE> struct CGSolve {
   using W = typename WideOf<T>::type;
   static constexpr bool CL = MODE == CG_CLUSTER;
@@ -470,12 +475,11 @@ template <typename T, int MODE> struct CGSolve {
   int rank, K;
   uint32_t dyn;   // address of the dynamic shared memory
 
-  // Barrier over a cluster: the hardware barrier (it does not spin; a budget below zero still
-  // gives up).
+  // Barrier over a cluster: the hardware barrier (it does not spin; in the cluster engine a budget
+  // below zero still gives up, at the first one, before anything is read through the cluster).
   __device__ bool cbar() const {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (q.c.budget < 0) {
+    cluster_barrier();
+    if (CL && q.c.budget < 0) {
       if (threadIdx.x == 0) atomicCAS(q.c.status, 0, 6);
       return false;
     }
@@ -483,6 +487,7 @@ template <typename T, int MODE> struct CGSolve {
   }
   // Barrier over all blocks of the solve: the arrival counter of grid_sync (a flag per block that
   // every block polls measured 2 to 5 us against its 1.3 us at 152 blocks: the polls' traffic).
+  // One that fails has failed in every block.
   __device__ bool bar() const {
     if constexpr (CL) return cbar();
     else return grid_sync(q.c);
@@ -880,28 +885,16 @@ enum { A_SUMF = 0, A_BB = 1, A_RR = 2, A_RU = 3, A_DU = 4, A_SUMX = 5, A_SLOTS =
 //   o = M^{-1} b, gamma = (r,o)                                        | barrier
 //   w = A o, p = o + beta p, s = w + beta s, delta = (w,o)             | barrier
 //   beta = gamma/gamma_old, a = gamma/(delta - beta gamma/a_old)
+// Returns early where a barrier failed.
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ idx, CGVec<T> v, T* __restrict__ wfull,
-                                                      Rhs<T> rhs, CGCtl2 q, MGP mg, CGGuess<T> gs) {
+__device__ __forceinline__ void cg_block(const int* __restrict__ idx, const CGVec<T>& v, T* __restrict__ wfull,
+                                         const Rhs<T>& rhs, const CGCtl2& q, const MGP& mg, const CGGuess<T>& gs,
+                                         unsigned char* cg_dyn, CGShared<T>& S) {
   using W = typename WideOf<T>::type;
   constexpr bool CL = MODE == CG_CLUSTER;
-  extern __shared__ __align__(16) unsigned char cg_dyn[];
-  __shared__ CGShared<T> S;
   const int rank = blockIdx.x, K = gridDim.x, t0 = threadIdx.x;
   const CGCtl& c = q.c;
-  if (t0 < (int)(sizeof(CGLayout) / 4)) reinterpret_cast<int*>(&S.lay)[t0] = reinterpret_cast<const int*>(q.lay)[t0];
-  const int skip = (q.sel & 2) ? q.other->bytes <= kCgSmem : 0;
-  const int st0 = *(volatile int*)c.status;   // an earlier failure (too many components, a lost copy): no solve
-  __syncthreads();
-  if (skip || st0 != 0 || ((q.sel & 1) && S.lay.bytes > kCgSmem)) return;
   const int M = S.lay.cnt[0];
-  if (M == 0) {
-    if (rank == 0 && t0 == 0) {
-      *c.iters = 0;
-      *c.resid = 0.0;
-    }
-    return;
-  }
   const uint32_t dyn = smem_u32(cg_dyn);
   const int na0 = S.lay.n[0], base = rank * na0;
   const int n0 = max(0, min(na0, M - base));
@@ -1278,7 +1271,31 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
     if (!conv) atomicCAS(c.status, 0, 5);
     atomicAdd(c.work, (unsigned long long)k * (unsigned long long)M);
   }
-  if constexpr (MODE != CG_GRID) A.cbar();   // no block leaves while another still reads its shared memory
+}
+
+template <typename T, int MODE>
+__global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ idx, CGVec<T> v, T* __restrict__ wfull,
+                                                      Rhs<T> rhs, CGCtl2 q, MGP mg, CGGuess<T> gs) {
+  extern __shared__ __align__(16) unsigned char cg_dyn[];
+  __shared__ CGShared<T> S;
+  const int t0 = threadIdx.x;
+  if (t0 < (int)(sizeof(CGLayout) / 4)) reinterpret_cast<int*>(&S.lay)[t0] = reinterpret_cast<const int*>(q.lay)[t0];
+  const int skip = (q.sel & 2) ? q.other->bytes <= kCgSmem : 0;
+  const int st0 = *(volatile int*)q.c.status;   // an earlier failure (too many components, a lost copy): no solve
+  __syncthreads();
+  if (skip || st0 != 0 || ((q.sel & 1) && S.lay.bytes > kCgSmem)) return;
+  if (S.lay.cnt[0] == 0) {
+    if (blockIdx.x == 0 && t0 == 0) {
+      *q.c.iters = 0;
+      *q.c.resid = 0.0;
+    }
+    return;
+  }
+  cg_block<T, MODE>(idx, v, wfull, rhs, q, mg, gs, cg_dyn, S);
+  // No block leaves while another of its cluster may still read its shared memory, after a failed
+  // barrier either: all of them fail at the same one, and one that has yet to arrive there may be
+  // reading those that wait.
+  if constexpr (MODE != CG_GRID) cluster_barrier();
 }
 
 // <w, f>: sum over the band (the nonlocal energy term).

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include "barrier.h"
 #include "fft.cuh"
 
 namespace etd {
@@ -963,8 +964,8 @@ __global__ void k_cg_setup(Geo g, ModelC<T> mc, const int* __restrict__ idx, con
                            const unsigned char* __restrict__ mask, const int* __restrict__ bmap,
                            const T* __restrict__ G, CGVec<T> v, int* cc_flags) {
   const int M = *count;
-  // labelling: component count, fallback flag, barrier counters of the fallback
-  if (blockIdx.x == 0 && threadIdx.x < 4) cc_flags[threadIdx.x] = 0;
+  // labelling: component count, fallback flag, the fallback's barrier word
+  if (blockIdx.x == 0 && threadIdx.x < 3) cc_flags[threadIdx.x] = 0;
   const int nd = g.nz > 1 ? 6 : 4;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
     const int p = idx[i];
@@ -1079,7 +1080,7 @@ struct CompAcc {
 };
 
 struct CGCtl {
-  unsigned* bar;        // [0] monotonic arrival count
+  unsigned* bar;        // the grid barrier's word
   int* status;          // plan status word
   int* iters;           // out: iterations
   double* resid;        // out: relative residual
@@ -1098,15 +1099,16 @@ struct CGCtl {
 // only valid for data that no thread writes during the launch.  The couplings, neighbour lists
 // and level maps are built by earlier launches and are read normally.
 
-// Grid-wide barrier for a cooperative launch on one monotonic arrival counter (zeroed
-// before the launch): barrier number e completes when the counter reaches e * gridDim.x,
-// and each block learns e from the value its own arrival returned, so nothing is reset
+// Grid-wide barrier for a cooperative launch on one word (barrier.h; zeroed before the launch):
+// each block learns its barrier from the value its own arrival returned, so nothing is reset
 // between barriers.  The block's writes are published by the block barrier followed by an
 // acquire-release add at GPU scope; blocks that arrive early poll with acquire loads, and
 // the last one to arrive takes its acquire from the add itself (without it, its L1 could
-// still hold lines that other blocks rewrote during the phase).  The spin has a
-// clock budget: when it runs out the kernel records ETD_ETIMEOUT in the status word and
-// every block returns at its next check.  Returns false once the status is non-zero.
+// still hold lines that other blocks rewrote during the phase).  The spin has a clock budget: a
+// block whose budget runs out, or (HEED) that finds the status word set by an earlier failure,
+// closes the word, and the barrier then fails in every block; one that was complete by then
+// passes in every block.  Returns false for a failed barrier, with the status word set
+// (ETD_ETIMEOUT unless something else was there).
 __device__ __forceinline__ unsigned atom_add_acq_rel_gpu(unsigned* p, unsigned v) {
   unsigned old;
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
@@ -1118,30 +1120,30 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   return v;
 }
 
-__device__ __forceinline__ bool grid_sync(const CGCtl& c) {
+template <bool HEED = true> __device__ __forceinline__ bool grid_sync(const CGCtl& c) {
   __syncthreads();
   __shared__ int ok;
   if (threadIdx.x == 0) {
     const unsigned nb = gridDim.x;
-    // the status word is read along with the counter, not after it (one L2 latency less); a
-    // failure that this misses is seen at the next barrier, whose poll looks at it too
-    int st = *(volatile int*)c.status;
+    // the status word is read along with the arrival, not after it (one L2 latency less)
+    const int st = HEED ? *(volatile int*)c.status : 0;
     const unsigned old = atom_add_acq_rel_gpu(c.bar, 1u);
-    const unsigned target = (old / nb + 1u) * nb;
-    if (old + 1u != target) {
+    const unsigned target = bar_target(old, nb);
+    unsigned w = old + 1u;
+    if (!bar_decided(w, target)) {
       const long long t0 = clock64();
-      for (;;) {
-        st = *(volatile int*)c.status;
-        if ((int)(ld_acquire_gpu(c.bar) - target) >= 0 || st != 0) break;
-        if (clock64() - t0 > c.budget) {
-          atomicCAS(c.status, 0, 6);
-          st = 6;
+      while (!bar_decided(w = ld_acquire_gpu(c.bar), target)) {
+        if (st != 0 || clock64() - t0 > c.budget) {
+          // the swap fails only where another block arrived or closed the word: look again
+          if (atomicCAS(c.bar, w, bar_closed(target)) != w) continue;
+          w = bar_closed(target);
           break;
         }
         __nanosleep(32);
       }
     }
-    ok = st == 0;
+    ok = bar_passed(w, target, nb);
+    if (!ok) atomicCAS(c.status, 0, 6);
   }
   __syncthreads();
   return ok;

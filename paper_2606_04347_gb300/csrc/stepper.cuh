@@ -363,8 +363,8 @@ template <typename T> class Stepper : public PlanBase {
     cc_parent_ = alloc<int>(g_.n);
     cc_cid_ = alloc<int>(g_.n);
     cc_comp_ = alloc<int>(g_.n);
-    ncomp_ = alloc<int>(4);   // component count, fallback flag of the labelling, its barrier counters
-    ETD_CUDA(cudaMemset(ncomp_, 0, 4 * sizeof(int)));
+    ncomp_ = alloc<int>(3);   // component count, fallback flag of the labelling, its barrier's word
+    ETD_CUDA(cudaMemset(ncomp_, 0, 3 * sizeof(int)));
     ccL_ = alloc<int>(kCCCoarse);
     csize_ = alloc<double>(kCompCap);
     csum_ = alloc<double>(2 * kCompCap);
@@ -390,7 +390,7 @@ template <typename T> class Stepper : public PlanBase {
     ETD_CUDA(cudaMemset(scal_, 0, sizeof(double) * S_COUNT));
     cg_part_ = alloc<double>(A_SLOTS * kCgMaxBlocks);
     cg_lay_ = alloc<CGLayout>(3);
-    bar_ = alloc<unsigned>(2);
+    bar_ = alloc<unsigned>(1);
     status_ = alloc<int>(1);
     flag_ = alloc<int>(1);
     cg_iters_ = alloc<int>(1);
@@ -903,7 +903,7 @@ template <typename T> class Stepper : public PlanBase {
     }
     q.KC = kCgCluster;
     timed(ETD_K_CG, 0.0, [&] {
-      if (first != CG_CLUSTER || second >= 0) ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
+      if (first != CG_CLUSTER || second >= 0) ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(*bar_), st_));
       for (int e : {first, second}) {
         if (e < 0) continue;
         q.sel = second < 0 ? 0 : (e == first ? 1 : 2);
@@ -1428,7 +1428,7 @@ template <typename T> class Stepper : public PlanBase {
     c.bar = bar_;
     c.status = status_;
     c.budget = wait_budget_;
-    ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(unsigned) * 2, st_));
+    ETD_CUDA(cudaMemsetAsync(bar_, 0, sizeof(*bar_), st_));
     auto k = k_lanczos<T>;
     // Nodes spread over all SMs before they fill blocks: the FP64 work of a node on 2 operations a
     // clock and SM, and block sums over as few warps as hold nodes (5852 nodes FP64, 8 steps: 3
