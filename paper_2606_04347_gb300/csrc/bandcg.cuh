@@ -1040,7 +1040,7 @@ __device__ __forceinline__ void cg_block(const int* __restrict__ idx, const CGVe
   const float w1 = mg.w1;
 
   // one band component: the plain mean; several: the mean of each (Sec. 2.1 per component)
-  const int C = c.ncomp ? *c.ncomp : 1;
+  const int C = *c.ncomp;
   CompAcc cacc{S.csh, c.csum, C};
   if (C > 1) {
     if (rank == 0)
@@ -1284,6 +1284,13 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
   const int st0 = *(volatile int*)q.c.status;   // an earlier failure (too many components, a lost copy): no solve
   __syncthreads();
   if (skip || st0 != 0 || ((q.sel & 1) && S.lay.bytes > kCgSmem)) return;
+  // A band without usable labels: reported by every solve on it (a frozen band's labels are made
+  // once, and the report of that launch is cleared with the call that returns it).
+  const int C = *q.c.ncomp;
+  if (C > kCompCap || C < 0) {
+    if (blockIdx.x == 0 && t0 == 0) atomicCAS(q.c.status, 0, C < 0 ? 6 : 8);
+    return;
+  }
   if (S.lay.cnt[0] == 0) {
     if (blockIdx.x == 0 && t0 == 0) {
       *q.c.iters = 0;

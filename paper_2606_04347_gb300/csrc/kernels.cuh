@@ -1031,6 +1031,9 @@ static __global__ void k_zero_left(const int* __restrict__ old_idx, const int* _
 // index to a smaller one, so each chase follows strictly decreasing indices and ends, and a
 // failed link means another thread made progress (each loop is bounded by the node count).
 constexpr int kCompCap = 4096;   // components the band solve supports (more: status 8)
+// Component count of a band whose labelling gave up: negative whatever the blocks that were still
+// counting add to it.
+constexpr int kNoComponents = -(1 << 30);
 
 __device__ __forceinline__ int cc_root(int* __restrict__ parent, int v) {
   int cur = __ldcg(parent + v);

@@ -373,13 +373,21 @@ static __global__ void __launch_bounds__(256) k_cc_union(const int* __restrict__
   __shared__ double sh[kCompShared];
   if (!*fallback) return;
   const int M = *count, t0 = blockIdx.x * blockDim.x + threadIdx.x, ns = gridDim.x * blockDim.x;
+  // An earlier failure does not stop the labelling (a frozen band is labelled once, for all the
+  // steps after that failure has been reported); a barrier of its own that gives up leaves no
+  // component count, which the solves report.
+  auto barrier = [&] {
+    const bool ok = grid_sync<false>(c);
+    if (!ok && t0 == 0) atomicExch(ncomp, kNoComponents);
+    return ok;
+  };
   for (int i = t0; i < M; i += ns) {
     int m = i;
 #pragma unroll
     for (int f = 0; f < 6; ++f) m = min(m, nb[f * cap + i]);
     parent[i] = m;
   }
-  if (!grid_sync(c)) return;
+  if (!barrier()) return;
   for (int i = t0; i < M; i += ns) {
 #pragma unroll
     for (int f = 0; f < 6; f += 2) {       // the + faces: every band edge is seen from one end
@@ -399,13 +407,13 @@ static __global__ void __launch_bounds__(256) k_cc_union(const int* __restrict__
       }
     }
   }
-  if (!grid_sync(c)) return;
+  if (!barrier()) return;
   for (int i = t0; i < M; i += ns) {
     const int r = cc_root(parent, i);
     parent[i] = r;
     if (r == i) cid[i] = atomicAdd(ncomp, 1);
   }
-  if (!grid_sync(c)) return;
+  if (!barrier()) return;
   const int C = *(volatile int*)ncomp;
   if (C > kCompCap) {
     if (t0 == 0) atomicCAS(c.status, 0, 8);
