@@ -1281,7 +1281,11 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int* __restrict__ id
   const int t0 = threadIdx.x;
   if (t0 < (int)(sizeof(CGLayout) / 4)) reinterpret_cast<int*>(&S.lay)[t0] = reinterpret_cast<const int*>(q.lay)[t0];
   const int skip = (q.sel & 2) ? q.other->bytes <= kCgSmem : 0;
-  const int st0 = *(volatile int*)q.c.status;   // an earlier failure (too many components, a lost copy): no solve
+  // An earlier failure (no convergence, a lost copy): no solve.  Nothing sets the word while a
+  // cluster's launch runs, so all of its threads read the same.  A block of the other engines may
+  // start after another one has given up, and its threads, or the blocks, would read different
+  // values: there the first grid barrier looks at it.
+  const int st0 = MODE == CG_CLUSTER ? *(volatile int*)q.c.status : 0;
   __syncthreads();
   if (skip || st0 != 0 || ((q.sel & 1) && S.lay.bytes > kCgSmem)) return;
   // A band without usable labels: reported by every solve on it (a frozen band's labels are made

@@ -167,3 +167,21 @@ def test_solve_that_gives_up_leaves_the_device_usable(monkeypatch, n, prec):
             assert np.linalg.norm(res) <= (1e-10 if prec == 0 else 1e-3) * np.linalg.norm(b)
         plan.close()
     assert gave_up.count(-1) == 4 and None not in gave_up
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [(32, 32, 32), (128, 128, 64), (128, 128, 128)])   # cluster, hybrid, grid engine
+def test_solves_after_a_failure_keep_its_report(n):
+    """A solve that does not converge sets the status word; the solves after it return at once, the
+    report is the first failure's, and the plan works on."""
+    p = wl.workload("c2", n=16)[0].replace(dim=3, n=n, model=0, precision=1, scheme=1, cg_rtol=1e-6, cg_maxit=2)
+    r = np.sqrt(sum(c ** 2 for c in wl.grid(n, p.half_len, 3)))
+    phi = torch.tensor(wl.tanh_profile(1.6 - r, 0.09) * np.ones(p.shape), dtype=torch.float32, device="cuda:0")
+    u = torch.tensor(np.random.default_rng(5).uniform(0.3, 0.7, size=p.shape), dtype=torch.float32, device="cuda:0")
+    plan = Plan(p)
+    for _ in range(2):
+        plan.step(phi, u, 3)
+        with pytest.raises(EtdError) as ei:
+            plan.step(None, u, 0, diag=True)
+        assert ei.value.code == 5
+        assert plan.step(None, u, 0, diag=True)["cg_iters_last"] == 2
