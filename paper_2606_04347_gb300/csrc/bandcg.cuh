@@ -424,9 +424,10 @@ template <typename T> struct CGShared {
   W ws[2][32];
   W gamma, alpha;         // written and read by one thread
   double bb, rr, tol2;
-  T a, bt, sc;
+  T a, bt, sc;            // sc: FP64, of the residual's FP32 copy; FP32, of the whole solve
+  float pre;
   double mean;
-  int go;
+  int go, range;
   double csh[kCompShared];
 };
 
@@ -1073,14 +1074,14 @@ __device__ __forceinline__ void cg_block(const int* __restrict__ idx, const CGVe
   }
   W bb(0), rr(0);
   __syncthreads();
+  const auto mean_of = [&](int i) {
+    if (C == 1) return W(S.mean);
+    const int ci = c.comp[base + i];
+    return W(__ldcg(c.csum + ci) / c.csize[ci]);
+  };
   {
-    const W meanf(S.mean);
     for (int i = t0; i < n0; i += kCgThreads) {
-      W mf = meanf;
-      if (C > 1) {
-        const int ci = c.comp[base + i];
-        mf = W(__ldcg(c.csum + ci) / c.csize[ci]);
-      }
+      const W mf = mean_of(i);
       const W b = W(R[i]) - mf;
       const T xi = X[i];
       T ax = 0;
@@ -1101,23 +1102,64 @@ __device__ __forceinline__ void cg_block(const int* __restrict__ idx, const CGVe
   A.post(bb, A_BB, nact);
   A.post(rr, A_RR, nact);
   if (!A.bar()) return;
-  if (A.scalar_warp()) {
+  const auto first_test = [&] {
+    if (!A.scalar_warp()) return;
     const W tb = A.total(A_BB), tr = A.total(A_RR);
-    if (A.scalar_lane()) {
-      const double bbs = wide_d(tb);
-      S.bb = bbs;
-      S.rr = wide_d(tr);
-      S.tol2 = c.rtol * c.rtol * bbs;
-      S.go = (bbs == 0.0 || S.rr <= S.tol2) ? 0 : 1;
-      // FP64: the power of two that takes |b| into [1, 2), for the FP32 copy of the residual
-      if constexpr (sizeof(T) == 8) {
-        int ex = 0;
-        frexp(sqrt(bbs), &ex);
-        S.sc = ldexp(1.0, max(-1000, min(1000, 1 - ex)));
-      }
+    if (!A.scalar_lane()) return;
+    const double bbs = wide_d(tb);
+    S.bb = bbs;
+    S.rr = wide_d(tr);
+    S.tol2 = c.rtol * c.rtol * bbs;
+    S.go = (bbs == 0.0 || S.rr <= S.tol2) ? 0 : 1;
+  };
+  first_test();
+  if (A.scalar_lane()) {
+    S.sc = 1;
+    if constexpr (sizeof(T) == 8) {
+      // the power of two that takes |b| into [1, 2), for the FP32 copy of the residual
+      int ex = 0;
+      frexp(sqrt(S.bb), &ex);
+      S.sc = ldexp(1.0, max(-1000, min(1000, 1 - ex)));
+    } else {
+      S.range = !(fmax(S.bb, S.rr) < 1e30) || S.bb < 1e-20;
+      S.pre = S.rr < 1.0 && S.bb < 1.0 ? 0x1p60f : 0x1p-30f;
     }
   }
   __syncthreads();
+  if constexpr (sizeof(T) == 4) {
+    // (b,b) has FP32's range: a right-hand side above some 1e15 or below 1e-10 is solved in units
+    // of a power of two near sum |b| + |r| (exact, and undone at the end)
+    if (S.range) {
+      const float pre = S.pre;
+      const auto b_of = [&](int i) { return W(wnear(rhs(idx[base + i]))) - mean_of(i); };
+      W l(0);
+      for (int i = t0; i < n0; i += kCgThreads) l = l + W(pre * fabsf(wnear(b_of(i)))) + W(pre * fabsf(R[i]));
+      A.post(l, A_SUMX, nact);
+      if (!A.bar()) return;
+      if (A.scalar_warp()) {
+        const double t = wide_d(A.total(A_SUMX)) / (double)pre;
+        // not finite: left alone; up by 2^60 at most, which leaves room for a large initial guess
+        if (A.scalar_lane() && t > 0.0 && t < 1e300) S.sc = ldexpf(1.0f, max(-126, min(60, -ilogb(t))));
+      }
+      __syncthreads();
+      const float sc = S.sc;
+      bb = rr = W(0);
+      for (int i = t0; i < n0; i += kCgThreads) {
+        const W b = b_of(i) * W(sc);
+        const float r = R[i] * sc;
+        X[i] *= sc;
+        R[i] = r;
+        bb = bb + b * b;
+        rr = rr + W(r) * W(r);
+        L0.put(V_E, i, w1 * L0.idg(i) * r);
+      }
+      A.post(bb, A_BB, nact);
+      A.post(rr, A_RR, nact);
+      if (!A.bar()) return;
+      first_test();
+      __syncthreads();
+    }
+  }
   bool conv = !S.go;
   int k = 0;
   if (!conv) {
@@ -1253,7 +1295,7 @@ __device__ __forceinline__ void cg_block(const int* __restrict__ idx, const CGVe
     if (A.scalar_lane()) S.mean = wide_d(t) / M;
   }
   __syncthreads();
-  const T mx = (T)S.mean;
+  const T mx = (T)S.mean, usc = (T)1 / S.sc;
   for (int i = t0; i < n0; i += kCgThreads) {
     const int p = idx[base + i];
     T mi = mx;
@@ -1261,7 +1303,8 @@ __device__ __forceinline__ void cg_block(const int* __restrict__ idx, const CGVe
       const int ci = c.comp[base + i];
       mi = (T)(__ldcg(c.csum + kCompCap + ci) / c.csize[ci]);
     }
-    const T w = X[i] - mi;
+    T w = X[i] - mi;
+    if constexpr (sizeof(T) == 4) w *= usc;
     wfull[p] = w;
     if (gs.hist) gs.hist[p] = w;
   }
