@@ -18,8 +18,11 @@
  *    2D.  Grid point (i,j,k) sits at (-X + i*hx, -Y + j*hy, -Z + k*hz), h = 2X/N (Sec. 2.1).
  *  - Element type is double for ETD_FP64 and float for ETD_FP32_MIXED.  FP32_MIXED keeps
  *    the phi-function tables (built in FP64, rounded once) and the scalar constraint terms in
- *    FP64, and every reduction (mass, volume, energy, CG dot products) in double-float (about
- *    48 bits) within a block, in FP64 across the mass, volume and energy sums' blocks.
+ *    FP64.  Its mass, volume and energy sums are compensated per thread and added in
+ *    double-float (about 48 bits, FP32's exponent range) within a block, in FP64 across the
+ *    blocks.  Its band solve sums a thread's nodes in FP32 (an iteration's dot products; up to
+ *    some hundred nodes) or double-float (the right-hand side, its norm and the first residual)
+ *    and adds the threads' and blocks' sums in double-float.
  *  - Field pointers are DEVICE pointers owned by the caller (for example PyTorch tensors
  *    on the plan's device).  They must stay valid until the enqueued work completes.  The
  *    library never frees them.  All work is enqueued on the stream given to etd_plan.
