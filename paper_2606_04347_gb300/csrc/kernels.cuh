@@ -247,12 +247,9 @@ template <typename T> struct EpiPhiG {
 // kappa/(mu eps^2) lambda in pass B.  Delta phi and grad phi are spectral (pass-A outputs).
 // V consecutive points per thread (16-byte loads and stores; V = 1 where u is not 16-byte
 // aligned), so that six wide loads a thread are in flight: 256^3 FP32 124 -> 88 us for 537 MB.
-// The FP64 form is bound by the FP64 pipe (70 instructions a point with its two quotients by
-// eps_phi and one by eps_u; 128^3 296 us) and multiplies by reciprocals instead.
-template <typename T> __device__ __forceinline__ T quot(T a, T b, T ib) {
-  if constexpr (sizeof(T) == 8) return a * ib;
-  else return a / b;
-}
+// The FP64 form is bound by the FP64 pipe (70 instructions a point with its quotients by eps_phi
+// and eps_u).  Products with reciprocals formed once would save 47 us a launch (128^3 coupled, three
+// steps: 18.80 ms a pass against 19.08), for one rounding more in each quotient: not taken.
 template <typename T, int V>
 __global__ void __launch_bounds__(256) k_r1(Geo g, ModelC<T> mc, const T* __restrict__ phi, const T* __restrict__ lap,
                      const T* __restrict__ gx, const T* __restrict__ gy, const T* __restrict__ gz,
@@ -260,7 +257,6 @@ __global__ void __launch_bounds__(256) k_r1(Geo g, ModelC<T> mc, const T* __rest
                      T* __restrict__ out_rest, T* __restrict__ out_wm) {
   using VT = VecN<T, V>;
   const T e = mc.eps_phi, e2 = e * e;
-  const T ie = (T)1 / e, ie2 = (T)1 / e2, ieu = (T)1 / mc.eps_u;
   const T dvol = (T)(hvol * scal[S_VOL] - scal[S_A0]);
   const T c_a = mc.kappa / (mc.mu * e2);
   const T c_b = mc.kappa / (mc.mu * e2 * e2);
@@ -289,17 +285,17 @@ __global__ void __launch_bounds__(256) k_r1(Geo g, ModelC<T> mc, const T* __rest
       const T Wp = dW(f), Wpp = d2W(f);
       const T Wm = Wp - mc.A1 * f;
       const T uu = uv.v[k];
-      T r = c_a * (Wpp - mc.A2) * (L - quot(mc.A1 * f, e2, ie2)) - (c_b * Wpp + c_c) * Wm;
+      T r = c_a * (Wpp - mc.A2) * (L - mc.A1 * f / e2) - (c_b * Wpp + c_c) * Wm;
       if (in_band(f, mc.band_hi)) {
         // line-tension term with Delta_{S,h} u (g = g(phi) at the faces), band points only
         const Nb n = neighbours(g, q * V + k);
         const T gzm = g.nz > 1 ? gloc(phi[n.zm]) : (T)0, gzp = g.nz > 1 ? gloc(phi[n.zp]) : (T)0;
         const T lu = surf_lap(g, mc, n, u, gloc(f), gloc(phi[n.xm]), gloc(phi[n.xp]), gloc(phi[n.ym]),
                               gloc(phi[n.yp]), gzm, gzp);
-        r += c_l * (mc.eps_u * lu - quot(gloc(f) * dW(uu), mc.eps_u, ieu)) * gn;
+        r += c_l * (mc.eps_u * lu - gloc(f) * dW(uu) / mc.eps_u) * gn;
       }
       r += c_v * gn;
-      r += c_al * (uu + mc.u0) * gn * (e * L - quot(Wp, e, ie));
+      r += c_al * (uu + mc.u0) * gn * (e * L - Wp / e);
       rv.v[k] = r;
       wv.v[k] = Wm;
     }
