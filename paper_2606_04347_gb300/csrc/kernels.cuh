@@ -656,12 +656,13 @@ struct EnergySum {   // sum of (a + b) d^2, or of a d, from FP32 values
     s.lo += __fmaf_rn(a, b, -t);
   }
 };
-template <typename T>
+// WIDE: FP64 sums also for FP32 storage, where the others left FP32's range (|u| from about 1e9).
+template <typename T, bool WIDE>
 __global__ void __launch_bounds__(256) k_energy_terms(Geo g, ModelC<T> mc, const T* __restrict__ G,
                                                       const T* __restrict__ U, const T* __restrict__ phi, double* scal) {
   double sg = 0, sw = 0, sm = 0, sv = 0;
   T mn = (T)INFINITY, mx = -(T)INFINITY;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (!WIDE) {
     EnergySum gx{}, gy{}, gz{}, w{};
     CompSum<float> m{}, v{};
     const Ubar<float> ub{mc.ubar, 0.0f};

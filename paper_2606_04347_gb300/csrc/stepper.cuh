@@ -124,12 +124,21 @@ template <typename T> class Stepper : public PlanBase {
     ETD_CUDA(cudaMemsetAsync(scal_ + S_GRAD, 0, sizeof(double) * 5, st_));
     double init[3] = {0.0, 1e300, -1e300};
     ETD_CUDA(cudaMemcpyAsync(scal_ + S_MAXB, init, sizeof(init), cudaMemcpyHostToDevice, st_));
-    k_energy_terms<T><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, Ge, U, ph, scal_);
+    k_energy_terms<T, sizeof(T) == 8><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, Ge, U, ph, scal_);
     k_band_dot<T><<<nsm_ * 4, 256, 0, st_>>>(idx_, count_, xe, rhs_gf(Ge, U), scal_ + S_NONLOC);
     ETD_CUDA(cudaGetLastError());
     ETD_CUDA(cudaStreamSynchronize(st_));
     double sc[S_COUNT];
     ETD_CUDA(cudaMemcpy(sc, scal_, sizeof(sc), cudaMemcpyDeviceToHost));
+    if (sizeof(T) == 4 && !std::isfinite(sc[S_GRAD] + sc[S_WELL] + sc[S_MASSF] + sc[S_VOLE])) {
+      // a term or a sum past FP32's range is an infinity or, in the compensation, a NaN
+      ETD_CUDA(cudaMemsetAsync(scal_ + S_GRAD, 0, sizeof(double) * 2, st_));   // S_GRAD, S_WELL
+      ETD_CUDA(cudaMemsetAsync(scal_ + S_MASSF, 0, sizeof(double) * 2, st_));  // S_MASSF, S_VOLE
+      k_energy_terms<T, true><<<grid_for(g_.n), 256, 0, st_>>>(g_, mc_, Ge, U, ph, scal_);
+      ETD_CUDA(cudaGetLastError());
+      ETD_CUDA(cudaStreamSynchronize(st_));
+      ETD_CUDA(cudaMemcpy(sc, scal_, sizeof(sc), cudaMemcpyDeviceToHost));
+    }
     int h[2];
     ETD_CUDA(cudaMemcpy(h, status_, sizeof(int), cudaMemcpyDeviceToHost));
     ETD_CUDA(cudaMemcpy(h + 1, count_, sizeof(int), cudaMemcpyDeviceToHost));

@@ -68,3 +68,28 @@ def test_step_of_an_unaligned_field():
     b = plan.step(phid, uu, 1, diag=True)
     assert abs(a["mass"] - b["mass"]) <= 1e-13 * abs(a["mass"])
     assert float((ud - uu).norm()) <= 1e-12 * float(ud.norm())
+
+
+@pytest.mark.parametrize("at", ["all", "one"])
+def test_energy_sums_past_fp32_range(at):
+    """Sums that leave FP32's range come out as the FP64 sums of the FP32 terms: |u| = 2e9, where
+    W(u) = 2.88e38 still fits FP32, at every point (the sums do not fit) or at one."""
+    p = _params((64, 32, 32), 1).replace(gamma=0.0, M=0.0, ubar=0.3)
+    rng = np.random.default_rng(8)
+    phi = _membrane(p, "full", rng).astype(np.float32).astype(np.float64)
+    u = np.full(p.shape, 2e9) if at == "all" else rng.uniform(0.2, 0.9, size=p.shape)
+    if at == "one":
+        u[7, 9, 11] = 2.1e9        # W(u) past FP32: infinite, as FP32 has it
+    u = u.astype(np.float32).astype(np.float64)
+    band, G = obm.band_mask(phi, p.band_mask_hi), omodel.g_loc(phi)
+    plan = Plan(p)
+    dev = lambda a: torch.tensor(a, dtype=torch.float32, device=DEV)  # noqa: E731
+    d = plan.energy(dev(phi), dev(u))
+    h3 = float(np.prod(p.h[:3]))
+    if at == "all":
+        want = h3 * float((G * 18.0 * (u * u - u) ** 2).sum()) / p.eps_u
+        assert abs(d["energy"] - want) <= 3e-6 * want
+    else:
+        assert d["energy"] == np.inf and d["umax"] == u.max()
+    mass = h3 * float((G * (3 * u * u - 2 * u ** 3 - p.ubar)).sum())
+    assert abs(d["mass"] - mass) <= 3e-6 * abs(mass)
