@@ -85,7 +85,7 @@ def aggregate(world: int, points: int, steps: int, ms_max: float) -> float:
     return world * points * steps / (ms_max / 1e3) / 1e6
 
 
-KERNEL_SOURCES = ("bandcg.cuh", "df32.cuh", "fft.cuh", "kernels.cuh", "ops.cuh")
+KERNEL_SOURCES = ("bandcg.cuh", "barrier.h", "df32.cuh", "fft.cuh", "kernels.cuh", "ops.cuh")
 
 
 def source_hash():

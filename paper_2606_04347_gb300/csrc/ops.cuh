@@ -48,8 +48,9 @@ __device__ __forceinline__ Row3<double> load_row(const double* t, int m) {
 __device__ __forceinline__ float4 load_row4(const float* t, int m) { return __ldg(reinterpret_cast<const float4*>(t) + m); }
 
 // Multipliers of the R values (kz = t + S r) that a lane of a row holds, by code: 0 identity, 1
-// Laplacian (lambda), 2..4 d/dx, d/dy, d/dz (i k, Nyquist -> 0).  The multiplier is chosen once, its x and y parts are the row's, and kz and |k|^2 are formed in T (integers below 2^24:
-// exact) instead of by a conversion per element and output.
+// Laplacian (lambda), 2..4 d/dx, d/dy, d/dz (i k, Nyquist -> 0).  The multiplier is chosen once,
+// its x and y parts are the row's, and kz and |k|^2 are formed in T (integers below 2^24: exact)
+// instead of by a conversion per element and output.
 template <typename T, int R, int S, typename C>
 __device__ __forceinline__ void deriv_row(int code, const C (&base)[R], C (&v)[R], const Wave& w, int t,
                                           const SpecConst<T>& k) {

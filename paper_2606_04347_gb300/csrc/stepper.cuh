@@ -1067,9 +1067,9 @@ template <typename T> class Stepper : public PlanBase {
   }
 
   // Coarse levels for the current band (level 0 = idx_, count_, mask_, bmap_, cg_).  Levels
-  // whose full grid has more than 2^15 cells use grid-wide kernels; the rest, the labels of the
-  // coarsest one are one launch of a single cluster (they are too small to
-  // fill the GPU, and launch gaps dominate).
+  // whose full grid has more than 2^15 cells use grid-wide kernels; the rest and the labels of
+  // the coarsest one are one launch of a single cluster (they are too small to fill the GPU, and
+  // launch gaps dominate).
   void mg_setup() {
     const int is3d = g_.nz > 1;
     int l = 1;
